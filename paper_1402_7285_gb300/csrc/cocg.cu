@@ -167,7 +167,7 @@ int run_solver(tb_ctx *ctx, const tb_bsr *H, const tb_bsr *S, const double *z, i
     // ---- workspace
     const size_t esz = mixed ? 4 : 8;
     const size_t vec_bytes = align_up(esz * 2 * n_rows * W, 256);
-    const int n_vec = (has_s ? 11 : 4) + (mixed ? 0 : 1); // + H p (recurrence) unless FP32
+    const int n_vec = mixed ? (has_s ? 11 : 4) : (has_s ? 9 : 2); // FP32: p twice and S p
     // df panels with S: the inner solve runs as FP32 sweeps with df refinement
     // (FP32 sweep residual, correction and product: three FP32 vectors)
     const bool ir = has_s && opts.precision == TB_PREC_DF64;
@@ -268,14 +268,18 @@ int run_solver(tb_ctx *ctx, const tb_bsr *H, const tb_bsr *S, const double *z, i
     int vi = 0;
     auto vec = [&]() { return (double *)(vb + vec_bytes * (vi++)); };
     p.RT = vec();
-    p.P[0] = vec();
-    p.P[1] = vec();
     p.U = vec();
-    p.HP = mixed ? nullptr : vec();
+    if (mixed) {
+        p.P[0] = vec();
+        p.P[1] = vec();
+    }
     if (has_s) {
         p.R[0] = vec();
         p.R[1] = vec();
-        p.SP = vec();
+        if (mixed)
+            p.SP = vec();
+        else
+            p.P[0] = vec();
         p.Tv = vec();
         p.D[0] = vec();
         p.D[1] = vec();

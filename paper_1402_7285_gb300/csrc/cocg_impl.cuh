@@ -58,16 +58,18 @@ __device__ __forceinline__ ShiftState fresh_shift() {
 }
 
 // A restarting column (a stall restart, or a slot that took the next column of
-// the queue) starts its recurrences again with beta = 0: its previous direction
-// and the vectors kept by recurrence are cleared, so that nothing of the old
+// the queue) starts its recurrences again with beta = 0: what it keeps by
+// recurrence (u and p; FP32 panels: p and S p) is cleared, so that nothing of the old
 // column (not even an inf or a NaN) survives the multiplication by zero.
 template <typename T, int W>
 __device__ __forceinline__ void clear_restart_row(const Panel<T> &p, int n, int64_t row, int col) {
     const int64_t o = (row * W + col) * 2;
-    T *pp = p.P[n & 1];
-    pp[o] = pp[o + 1] = (T)0;
-    if (p.SP) p.SP[o] = p.SP[o + 1] = (T)0;
-    if (p.HP) p.HP[o] = p.HP[o + 1] = (T)0;
+    T *pp = p.P[1] ? p.P[n & 1] : p.P[0]; // FP32 panels alternate between two buffers
+    if (pp) pp[o] = pp[o + 1] = (T)0;
+    if (p.SP)
+        p.SP[o] = p.SP[o + 1] = (T)0;
+    else
+        p.U[o] = p.U[o + 1] = (T)0; // alpha is 0 in this iteration: u is not used any more
 }
 
 template <typename T, int W>
@@ -101,19 +103,18 @@ __global__ void k_init_vec(Panel<T> p, int64_t n_rows, int has_s) {
         const T one = (j == row) ? (T)1 : (T)0;
         const int64_t o = t * 2;
         p.RT[o] = one, p.RT[o + 1] = 0;
-        p.P[0][o] = p.P[0][o + 1] = 0;
-        p.P[1][o] = p.P[1][o + 1] = 0;
+        if (p.P[0]) p.P[0][o] = p.P[0][o + 1] = 0;
+        if (p.P[1]) p.P[1][o] = p.P[1][o + 1] = 0;
         p.U[o] = p.U[o + 1] = 0;
         if (has_s) {
             p.R[0][o] = p.R[0][o + 1] = 0;
             p.R[1][o] = one, p.R[1][o + 1] = 0;
-            p.SP[o] = p.SP[o + 1] = 0;
+            if (p.SP) p.SP[o] = p.SP[o + 1] = 0;
             p.Tv[o] = p.Tv[o + 1] = 0;
             p.D[0][o] = p.D[0][o + 1] = 0;
             p.D[1][o] = p.D[1][o + 1] = 0;
             p.Av[o] = p.Av[o + 1] = 0;
         }
-        if (p.HP) p.HP[o] = p.HP[o + 1] = 0;
     }
     const int64_t ne = (int64_t)W * p.max_col_ent * p.nz;
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < ne; t += stride) {
@@ -347,25 +348,25 @@ __global__ void __launch_bounds__(NT, (B <= 4 ? 3 : 1)) k_outer(Panel<T> p) {
     using TM = Teams<T, W, NT>;
     constexpr int CPT = TM::CPT;
     const int team = threadIdx.x / TM::TPR, lane = threadIdx.x % TM::TPR;
-    // H p_n: with FP64 and df panels, H r_n + beta_{n-1} (H p_{n-1}) (one
-    // product of the finished r_n, H p kept by this recurrence, so the product
-    // reads plain neighbour rows); with FP32 panels, the product of p_n formed
-    // on the fly from r_n and p_{n-1}.
-    constexpr bool HP_REC = !std::is_same<T, float>::value;
+    // FP64 and df panels keep u = (z_s S - H) p_n by recurrence, u_n = z_s rt_n -
+    // H r_n + beta u_{n-1}, so no S p or H p is stored and the product reads
+    // finished rows.  S = I: mu_n = p_n^T u_n = r_n^T u_n (p_{n-1}^T u_n = 0), no p
+    // either: r and u in, u out, 3 panel vectors instead of 6.  With S, r = S^-1 rt
+    // carries the inner solve's error, with which r^T u costs up to 30 % more
+    // iterations (the p^T u form 4 %), so p is kept: 6 vectors instead of 9.
+    // FP32 panels form p_n on the fly and multiply it.
+    constexpr bool U_REC = !std::is_same<T, float>::value;
     const int n = p.ctl->n;
     const T *Rc = HAS_S ? p.R[n & 1] : p.RT;
-    T *Pnew = p.P[n & 1];
-    LdAxpy<T, W> ld; // p_n = r_n + beta_{n-1} p_{n-1}
+    LdAxpy<T, W> ld; // p_n = r_n + beta_{n-1} p_{n-1}; r_n when u is kept by recurrence
     ld.a = Rc;
-    ld.b = p.P[(n + 1) & 1];
+    ld.b = U_REC ? nullptr : p.P[(n + 1) & 1];
     ld.lane = lane;
 #pragma unroll
     for (int cc = 0; cc < CPT; ++cc) {
         const ColState &C = p.col[lane * CPT + cc];
         ld.s[cc] = C.done ? mk<T>(0, 0) : cvt<T>(C.beta_prev);
     }
-    LdAxpy<T, W> lr = ld; // r_n
-    lr.b = nullptr;
     cpx<T> zs[CPT]; // each column's seed shift
 #pragma unroll
     for (int cc = 0; cc < CPT; ++cc) zs[cc] = cvt<T>(p.col[lane * CPT + cc].zs);
@@ -375,36 +376,44 @@ __global__ void __launch_bounds__(NT, (B <= 4 ? 3 : 1)) k_outer(Panel<T> p) {
     const int64_t br_step = (int64_t)gridDim.x * TM::PER_CTA; // groups dealt round-robin
     for (int64_t br = (int64_t)blockIdx.x * TM::PER_CTA + team; br < p.n_brows; br += br_step) {
         cpx<T> y[B][CPT];
-        if constexpr (HP_REC)
-            bsr_row_product<T, B>(p.h_rp, p.h_ci, p.h_val, br, lr, y);
-        else
-            bsr_row_product<T, B>(p.h_rp, p.h_ci, p.h_val, br, ld, y);
+        bsr_row_product<T, B>(p.h_rp, p.h_ci, p.h_val, br, ld, y);
 #pragma unroll
         for (int i = 0; i < B; ++i) {
             const int64_t row = br * B + i;
-            cpx<T> pv[CPT], u[CPT];
+            cpx<T> pv[CPT], u[CPT]; // p_n (r_n when S = I); u_n
             ld(row, pv);
-            st_row<T, W>(Pnew, row, lane, pv);
-            if constexpr (HP_REC) {
-                cpx<T> hp[CPT];
-                ld_row<T, W>(p.HP, row, lane, hp);
+            if constexpr (U_REC) {
+                cpx<T> rt[CPT];
+                ld_row<T, W>(p.U, row, lane, u);
+                if constexpr (HAS_S) {
+                    cpx<T> po[CPT];
+                    ld_row<T, W>(p.P[0], row, lane, po);
+                    ld_row<T, W>(p.RT, row, lane, rt);
 #pragma unroll
-                for (int cc = 0; cc < CPT; ++cc) y[i][cc] = y[i][cc] + ld.s[cc] * hp[cc];
-                st_row<T, W>(p.HP, row, lane, y[i]);
-            }
-            if constexpr (HAS_S) {
-                cpx<T> rt[CPT], sp[CPT];
-                ld_row<T, W>(p.RT, row, lane, rt);
-                ld_row<T, W>(p.SP, row, lane, sp);
+                    for (int cc = 0; cc < CPT; ++cc) pv[cc] = pv[cc] + ld.s[cc] * po[cc];
+                    st_row<T, W>(p.P[0], row, lane, pv);
+                } else {
 #pragma unroll
-                for (int cc = 0; cc < CPT; ++cc) {
-                    sp[cc] = rt[cc] + ld.s[cc] * sp[cc];
-                    u[cc] = zs[cc] * sp[cc] - y[i][cc];
+                    for (int cc = 0; cc < CPT; ++cc) rt[cc] = pv[cc];
                 }
-                st_row<T, W>(p.SP, row, lane, sp);
-            } else {
 #pragma unroll
-                for (int cc = 0; cc < CPT; ++cc) u[cc] = zs[cc] * pv[cc] - y[i][cc];
+                for (int cc = 0; cc < CPT; ++cc) u[cc] = (zs[cc] * rt[cc] - y[i][cc]) + ld.s[cc] * u[cc];
+            } else {
+                st_row<T, W>(p.P[n & 1], row, lane, pv);
+                if constexpr (HAS_S) {
+                    cpx<T> rt[CPT], sp[CPT];
+                    ld_row<T, W>(p.RT, row, lane, rt);
+                    ld_row<T, W>(p.SP, row, lane, sp);
+#pragma unroll
+                    for (int cc = 0; cc < CPT; ++cc) {
+                        sp[cc] = rt[cc] + ld.s[cc] * sp[cc];
+                        u[cc] = zs[cc] * sp[cc] - y[i][cc];
+                    }
+                    st_row<T, W>(p.SP, row, lane, sp);
+                } else {
+#pragma unroll
+                    for (int cc = 0; cc < CPT; ++cc) u[cc] = zs[cc] * pv[cc] - y[i][cc];
+                }
             }
             st_row<T, W>(p.U, row, lane, u);
 #pragma unroll
@@ -1221,7 +1230,7 @@ struct SolveLaunch {
         f.R[0] = f.R[1] = p.C32;
         f.Tv = p.T32;
         f.Av = p.A32;
-        f.RT = f.P[0] = f.P[1] = f.SP = f.U = f.HP = nullptr;
+        f.RT = f.P[0] = f.P[1] = f.SP = f.U = nullptr;
         for (int k = 0; k < 2; ++k) f.D[k] = reinterpret_cast<float *>(p.D[k]);
         return f;
     }
