@@ -7,10 +7,10 @@ __global__ void k_copy_z(const double *z, c64 *zc, int nz) {
     for (int i = threadIdx.x; i < nz; i += blockDim.x) zc[i] = mk(z[2 * i], z[2 * i + 1]);
 }
 
-// *not_unit = 1 unless every block row holds a diagonal block equal to the
-// identity (the overlap of orthonormal orbitals on one site).
+// Result (check_words) 1 unless every block row holds a diagonal block equal to
+// the identity (the overlap of orthonormal orbitals on one site).
 __global__ void k_unit_diag(const int64_t *rp, const int32_t *ci, const double *val, int64_t n_brows, int b,
-                            int *not_unit) {
+                            int *words, int *host) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t br = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; br < n_brows; br += stride) {
         bool ok = false;
@@ -20,8 +20,9 @@ __global__ void k_unit_diag(const int64_t *rp, const int32_t *ci, const double *
             for (int q = 0; q < b * b; ++q)
                 if (val[k * b * b + q] != ((q / b == q % b) ? 1.0 : 0.0)) ok = false;
         }
-        if (!ok) atomicOr(not_unit, 1);
+        if (!ok) atomicOr(words, 1);
     }
+    publish_check(words, host);
 }
 
 } // namespace tbgf
@@ -152,15 +153,13 @@ int run_solver(tb_ctx *ctx, const tb_bsr *H, const tb_bsr *S, const double *z, i
     if (rc) return rc;
     int s_unit = 0;
     if (has_s) {
-        int *flag = nullptr;
-        TB_CUDA_TRY(ctx, cudaMallocAsync((void **)&flag, sizeof(int), stream));
-        TB_CUDA_TRY(ctx, cudaMemsetAsync(flag, 0, sizeof(int), stream));
+        int *words = nullptr, *host = nullptr, h = 1;
+        rc = check_words(ctx, &words, &host);
+        if (rc) return rc;
         k_unit_diag<<<num_sms() * 4, 256, 0, stream>>>((const int64_t *)d_srp, (const int32_t *)d_sci,
-                                                      (const double *)d_sval, S->n_brows, b, flag);
-        int h = 1;
-        TB_CUDA_TRY(ctx, cudaMemcpyAsync(&h, flag, sizeof(int), cudaMemcpyDeviceToHost, stream));
-        TB_CUDA_TRY(ctx, cudaFreeAsync(flag, stream));
-        TB_CUDA_TRY(ctx, cudaStreamSynchronize(stream));
+                                                      (const double *)d_sval, S->n_brows, b, words, host);
+        rc = check_wait(ctx, stream, &h);
+        if (rc) return rc;
         s_unit = h == 0;
     }
 

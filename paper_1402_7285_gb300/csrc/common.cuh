@@ -74,6 +74,11 @@ struct tb_ctx {
     // grow-only device workspace slots owned by the context
     std::vector<void *> ws_ptr;
     std::vector<size_t> ws_size;
+    // structure checks: device words (bits found so far, arrival counter, result)
+    // and the host copy of the result that the checking kernel writes
+    int *chk_dev = nullptr;
+    volatile int *chk_host = nullptr;
+    cudaEvent_t chk_ev = nullptr;
 };
 
 namespace tbgf {
@@ -141,13 +146,38 @@ class Stager {
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
-// Checks a device BSR structure (row_ptr monotone from 0 to nnzb, col_idx in
-// range and ascending within each block row) and the 16-byte alignment of its
-// values; returns TB_OK or TB_ERR_STRUCTURE / TB_ERR_ARG.  Synchronises `s`.
-// Structure check of validate_bsr as a kernel: ORs 1 into *bad for a bad
-// row pointer, 2 for a column index out of range or out of order.
+// Structure check of a device BSR matrix by one block row: 1 for a bad row
+// pointer, 2 for a column index out of range or out of order, else 0.
+__device__ __forceinline__ int bsr_row_fault(const int64_t *rp, const int32_t *ci, int64_t n_brows, int64_t nnzb,
+                                             int64_t a) {
+    const int64_t k0 = rp[a], k1 = rp[a + 1];
+    if (k0 > k1 || k0 < 0 || k1 > nnzb || (a == 0 && k0 != 0) || (a == n_brows - 1 && k1 != nnzb)) return 1;
+    int64_t prev = -1;
+    for (int64_t k = k0; k < k1; ++k) {
+        const int64_t c = ci[k];
+        if (c < 0 || c >= n_brows || c <= prev) return 2;
+        prev = c;
+    }
+    return 0;
+}
+
+// The check as a kernel: ORs the faults of all block rows into *bad.
 __global__ void k_validate_bsr(const int64_t *rp, const int32_t *ci, int64_t n_brows, int64_t nnzb, int *bad);
 
+// A checking kernel's result reaches the host without an allocation, a memset or
+// a copy: check_words() gives (once per context) three device words and a pinned
+// host word; the kernel ORs what it finds into words[0] and its last CTA calls
+// publish_check, which writes the result to words[2] (for kernels queued behind
+// it) and to the host word, and clears the others for the next check.
+// check_wait() records an event behind the kernel, waits for it and returns the
+// result.  (cudaMallocAsync + memset + copy + cudaFreeAsync with the default
+// pool, which gives its memory back at every synchronisation, took 190 us.)
+int check_words(tb_ctx *ctx, int **words, int **host);
+int check_wait(tb_ctx *ctx, cudaStream_t s, int *result);
+
+// Checks a device BSR structure (row_ptr monotone from 0 to nnzb, col_idx in
+// range and ascending within each block row) and the 16-byte alignment of its
+// values; returns TB_OK or TB_ERR_STRUCTURE / TB_ERR_ARG.  Waits for the check.
 int validate_bsr(tb_ctx *ctx, const int64_t *row_ptr, const int32_t *col_idx, const void *val, int64_t n_brows,
                  int64_t nnzb, cudaStream_t s, const char *name);
 
@@ -176,4 +206,14 @@ __device__ __forceinline__ bool last_cta_arrival(unsigned int *counter) {
     __syncthreads();
     if (is_last) __threadfence();
     return is_last != 0;
+}
+
+// The end of a checking kernel (see check_words): every thread of every CTA calls it.
+__device__ __forceinline__ void publish_check(int *words, int *host) {
+    if (last_cta_arrival(reinterpret_cast<unsigned int *>(words + 1)) && threadIdx.x == 0) {
+        const int r = atomicExch(words, 0);
+        words[2] = r;
+        *reinterpret_cast<volatile int *>(host) = r;
+        __threadfence_system();
+    }
 }

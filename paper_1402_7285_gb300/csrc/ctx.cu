@@ -98,22 +98,48 @@ int Stager::finish() {
 
 __global__ void k_validate_bsr(const int64_t *rp, const int32_t *ci, int64_t n_brows, int64_t nnzb, int *bad) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < n_brows; a += stride) {
-        const int64_t k0 = rp[a], k1 = rp[a + 1];
-        if (k0 > k1 || k0 < 0 || k1 > nnzb || (a == 0 && k0 != 0) || (a == n_brows - 1 && k1 != nnzb)) {
-            atomicOr(bad, 1);
-            continue;
+    for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < n_brows; a += stride)
+        if (const int f = bsr_row_fault(rp, ci, n_brows, nnzb, a)) atomicOr(bad, f);
+}
+
+static __global__ void k_check_bsr(const int64_t *rp, const int32_t *ci, int64_t n_brows, int64_t nnzb, int *words,
+                                   int *host) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < n_brows; a += stride)
+        if (const int f = bsr_row_fault(rp, ci, n_brows, nnzb, a)) atomicOr(words, f);
+    publish_check(words, host);
+}
+
+int check_words(tb_ctx *ctx, int **words, int **host) {
+    if (!ctx->chk_dev) {
+        int *d = nullptr;
+        TB_CUDA_TRY(ctx, cudaMalloc((void **)&d, 4 * sizeof(int)));
+        cudaError_t e = cudaMemset(d, 0, 4 * sizeof(int));
+        if (e == cudaSuccess) e = cudaHostAlloc((void **)&ctx->chk_host, sizeof(int), cudaHostAllocPortable);
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->chk_ev, cudaEventDisableTiming);
+        // the memset ran on the legacy stream, which a caller's non-blocking stream does not wait for
+        if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
+        if (e != cudaSuccess) {
+            cudaFree(d);
+            if (ctx->chk_host) cudaFreeHost((void *)ctx->chk_host);
+            if (ctx->chk_ev) cudaEventDestroy(ctx->chk_ev);
+            ctx->chk_host = nullptr;
+            ctx->chk_ev = nullptr;
+            return set_error(ctx, TB_ERR_CUDA, "structure check words: %s", cudaGetErrorString(e));
         }
-        int64_t prev = -1;
-        for (int64_t k = k0; k < k1; ++k) {
-            const int64_t c = ci[k];
-            if (c < 0 || c >= n_brows || c <= prev) {
-                atomicOr(bad, 2);
-                break;
-            }
-            prev = c;
-        }
+        ctx->chk_dev = d;
     }
+    *words = ctx->chk_dev;
+    *host = (int *)ctx->chk_host;
+    return TB_OK;
+}
+
+int check_wait(tb_ctx *ctx, cudaStream_t s, int *result) {
+    TB_CUDA_TRY(ctx, cudaGetLastError());
+    TB_CUDA_TRY(ctx, cudaEventRecord(ctx->chk_ev, s));
+    TB_CUDA_TRY(ctx, cudaEventSynchronize(ctx->chk_ev));
+    *result = *ctx->chk_host;
+    return TB_OK;
 }
 
 int validate_bsr(tb_ctx *ctx, const int64_t *row_ptr, const int32_t *col_idx, const void *val, int64_t n_brows,
@@ -121,15 +147,13 @@ int validate_bsr(tb_ctx *ctx, const int64_t *row_ptr, const int32_t *col_idx, co
     if (((uintptr_t)val & 15u) != 0)
         return set_error(ctx, TB_ERR_ARG, "%s values must be 16-byte aligned", name);
     if (n_brows <= 0 || nnzb < 0) return set_error(ctx, TB_ERR_STRUCTURE, "%s: bad sizes", name);
-    int *flag = nullptr;
-    TB_CUDA_TRY(ctx, cudaMallocAsync((void **)&flag, sizeof(int), s));
-    TB_CUDA_TRY(ctx, cudaMemsetAsync(flag, 0, sizeof(int), s));
+    int *words = nullptr, *host = nullptr, h = 0;
+    int rc = check_words(ctx, &words, &host);
+    if (rc) return rc;
     const int g = (int)std::min<int64_t>((n_brows + 255) / 256, 152 * 8);
-    k_validate_bsr<<<g < 1 ? 1 : g, 256, 0, s>>>(row_ptr, col_idx, n_brows, nnzb, flag);
-    int h = 0;
-    TB_CUDA_TRY(ctx, cudaMemcpyAsync(&h, flag, sizeof(int), cudaMemcpyDeviceToHost, s));
-    TB_CUDA_TRY(ctx, cudaFreeAsync(flag, s));
-    TB_CUDA_TRY(ctx, cudaStreamSynchronize(s));
+    k_check_bsr<<<g < 1 ? 1 : g, 256, 0, s>>>(row_ptr, col_idx, n_brows, nnzb, words, host);
+    rc = check_wait(ctx, s, &h);
+    if (rc) return rc;
     if (h) return set_error(ctx, TB_ERR_STRUCTURE, "%s: malformed BSR structure (code %d)", name, h);
     return TB_OK;
 }
@@ -162,6 +186,11 @@ int tb_ctx_destroy(tb_ctx *ctx) {
     cudaDeviceSynchronize();
     for (void *p : ctx->ws_ptr)
         if (p) cudaFree(p);
+    if (ctx->chk_dev) {
+        cudaFree(ctx->chk_dev);
+        cudaFreeHost((void *)ctx->chk_host);
+        cudaEventDestroy(ctx->chk_ev);
+    }
     if (dev >= 0 && dev != ctx->device) cudaSetDevice(dev);
     delete ctx;
     return TB_OK;
