@@ -1,7 +1,8 @@
 // shifted_cocg_solve / shifted_cocg_profile: host driver of the panel shifted COCG.
-#include "cocg_impl.cuh"
+#include "engine.cuh"
 
 namespace tbgf {
+
 
 __global__ void k_copy_z(const double *z, c64 *zc, int nz) {
     for (int i = threadIdx.x; i < nz; i += blockDim.x) zc[i] = mk(z[2 * i], z[2 * i + 1]);
@@ -66,7 +67,7 @@ int fetch_host(tb_ctx *ctx, const X *p, size_t n, std::vector<X> &out) {
 int run_solver(tb_ctx *ctx, const tb_bsr *H, const tb_bsr *S, const double *z, int32_t n_z,
                const int64_t *rhs_rows, int64_t n_rhs, const int64_t *out_row_ptr, const int64_t *out_rows,
                const tb_solve_opts *opts_in, double *G, int32_t *iters, double *resid, int32_t *status,
-               int profile_reps, double *ms) {
+               int profile_reps, double *ms, bool graph_path = false) {
     if (!ctx) return TB_ERR_ARG;
     tb_solve_opts opts;
     if (opts_in)
@@ -119,8 +120,6 @@ int run_solver(tb_ctx *ctx, const tb_bsr *H, const tb_bsr *S, const double *z, i
 
     // ---- one panel of W slots; the columns form a queue in the given order: a
     // slot whose column finishes takes the next column (refill on the device)
-    int W = opts.panel_w;
-    if (W == 0) W = panel_width_for((int)std::min<int64_t>(n_rhs, mixed ? 64 : 32));
     int64_t max_col_ent = 1;
     for (int64_t c = 0; c < n_rhs; ++c) max_col_ent = std::max<int64_t>(max_col_ent, h_optr[c + 1] - h_optr[c]);
     TB_CHECK(ctx, max_col_ent < (1 << 24), TB_ERR_SIZE, "too many kept rows in one column");
@@ -163,15 +162,46 @@ int run_solver(tb_ctx *ctx, const tb_bsr *H, const tb_bsr *S, const double *z, i
         s_unit = h == 0;
     }
 
+    // inner tolerance: FP64 and FP32 panels 1e-3 tol (floors 1e-13, 1e-7); df panels
+    // refine to 1e-5 tol (floor 1e-12): the refinement makes the tighter target cheap,
+    // and inexact inner solves are what separates the shifted results from the FP64 ones
+    const bool dfs = has_s && opts.precision == TB_PREC_DF64;
+    const double inner_tol = opts.inner_tol > 0.0 ? opts.inner_tol
+                                                  : (dfs ? std::max(1e-5 * opts.tol, 1e-12)
+                                                         : std::max(1e-3 * opts.tol, mixed ? 1e-7 : (lowp ? 1e-12 : 1e-13)));
+    const int inner_max = opts.inner_max > 0 ? opts.inner_max : 40;
+    // ---- FP64 and df panels run in the persistent kernel (engine.cuh) when S = I or the spectrum of S allows
+    // short Chebyshev sweeps; FP32 panels and other S (a wide spectrum, not positive definite) as a graph with
+    // conjugate gradients on S
+    Engine<double> en;
+    std::memset(&en, 0, sizeof(en));
+    bool engine = !mixed && !graph_path;
+    if (engine && has_s) {
+        double lo = 1, hi = 0;
+        rc = spectral_bounds(ctx, (const int64_t *)d_srp, (const int32_t *)d_sci, (const double *)d_sval, S->n_brows, b,
+                             num_sms(), stream, &lo, &hi);
+        if (rc) return rc;
+        engine = chebyshev_terms(lo, hi, inner_tol, inner_max, lowp, en);
+    }
+    // slots: the panel width asked for, or 64 (the graph: the next compiled width up to 32, FP32 64); the persistent
+    // kernel takes any number, and then no more than there are columns.  C2 (131072 rows, df64, 64 columns): 64 slots
+    // solve a column in 14 % less time than 32.
+    int W = opts.panel_w;
+    if (engine)
+        W = W > 0 ? W : (int)std::min<int64_t>(n_rhs, MAX_W);
+    else if (W == 0)
+        W = panel_width_for((int)std::min<int64_t>(n_rhs, mixed ? 64 : 32));
+
     // ---- workspace
     const size_t esz = mixed ? 4 : 8;
     const size_t vec_bytes = align_up(esz * 2 * n_rows * W, 256);
-    const int n_vec = mixed ? (has_s ? 11 : 4) : (has_s ? 9 : 2); // FP32: p twice and S p
-    // df panels with S: the inner solve runs as FP32 sweeps with df refinement
-    // (FP32 sweep residual, correction and product: three FP32 vectors)
-    const bool ir = has_s && opts.precision == TB_PREC_DF64;
+    // FP32: p twice and S p; the persistent kernel: rt, u, p and (S) r, t
+    const int n_vec = engine ? (has_s ? 5 : 3) : mixed ? (has_s ? 11 : 4) : (has_s ? 9 : 2);
+    // FP32 sweeps with refinement (the persistent kernel, and df panels of the graph): three FP32
+    // vectors (sweep residual and two iterates; or residual, correction and product)
+    const bool ir = has_s && (engine || opts.precision == TB_PREC_DF64);
     const size_t vec32_bytes = align_up(sizeof(float) * 2 * n_rows * W, 256);
-    const int per_cta = NT / (W / (mixed ? 2 : 1));
+    const int per_cta = std::max(1, NT / (W / (mixed ? 2 : 1)));
     TB_CHECK(ctx, opts.ctas_per_sm >= 0 && opts.ctas_per_sm <= 8, TB_ERR_ARG, "ctas_per_sm must be 0..8");
     const int per_sm = opts.ctas_per_sm > 0 ? opts.ctas_per_sm : 3;
     int ncta = (int)std::min<int64_t>((int64_t)per_sm * num_sms(), (H->n_brows + per_cta - 1) / per_cta);
@@ -180,7 +210,7 @@ int run_solver(tb_ctx *ctx, const tb_bsr *H, const tb_bsr *S, const double *z, i
     // than the other kernels
     int ncta_a = ncta;
     // the FP32 sweep kernels of the refinement: FP32 team geometry (two complex per thread)
-    const int per_cta_f = NT / (W / 2);
+    const int per_cta_f = std::max(1, NT / std::max(1, W / 2));
     const int ncta_f = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)per_sm * num_sms(),
                                                                    (H->n_brows + per_cta_f - 1) / per_cta_f));
     // (with the refinement, df panels use IC_A only in FP32, and C was measured faster on the
@@ -192,9 +222,15 @@ int run_solver(tb_ctx *ctx, const tb_bsr *H, const tb_bsr *S, const double *z, i
     // (measured 70.9 against 72.5 us on C2 at W = 64)
     const int ncta_fb = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)std::max(1, per_sm - 1) * num_sms(),
                                                                     (H->n_brows + per_cta_f - 1) / per_cta_f));
-    const int ncta_max = std::max(std::max(ncta, ncta_a), ncta_f);
+    const int ncta_max = std::max(std::max(std::max(ncta, ncta_a), ncta_f), engine ? num_sms() * 8 : 0);
     void *vec_base = nullptr;
     rc = ws_get(ctx, WS_SOLVE_VEC, vec_bytes * n_vec + (ir ? 3 * vec32_bytes : 0), &vec_base);
+    if (rc == TB_ERR_ALLOC && engine && opts.panel_w == 0 && W > 32) { // half the slots where 64 do not fit
+        tb_solve_opts o = opts;
+        o.panel_w = 32;
+        return run_solver(ctx, H, S, z, n_z, rhs_rows, n_rhs, out_row_ptr, out_rows, &o, G, iters, resid, status,
+                          profile_reps, ms);
+    }
     if (rc) return rc;
     size_t off = 0;
     auto take = [&](size_t bytes) {
@@ -205,14 +241,19 @@ int run_solver(tb_ctx *ctx, const tb_bsr *H, const tb_bsr *S, const double *z, i
     const size_t o_col = take(sizeof(ColState) * W);
     const size_t o_sh = take(sizeof(ShiftState) * (size_t)W * n_z);
     const size_t o_ctl = take(sizeof(Ctrl));
-    const size_t o_part = take(sizeof(double) * (size_t)W * 4 * ncta_max);
+    const size_t o_bar = take(sizeof(GridBarrier));
+    const size_t o_sc = take(sizeof(SlotScalars<double>) * MAX_W);
+    // partial sums (the persistent kernel: 3 per slot and CTA, and 3 per slot and group of CTAs)
+    const size_t o_part = take(sizeof(double) * (size_t)(engine ? MAX_W : W) * 4 * ncta_max);
     const size_t o_zc = take(sizeof(c64) * n_z);
     const size_t o_crow = take(sizeof(int64_t) * n_rhs);
     const size_t o_cptr = take(sizeof(int64_t) * (n_rhs + 1));
     const size_t o_erow = take(sizeof(int64_t) * std::max<int64_t>(n_out, 1));
     const size_t o_stats = take(sizeof(int64_t) * 4);
     // many kept rows: the shifted steps' kept-row updates run row-parallel (k_rows_A / k_rows_B)
-    const bool rowpar = max_col_ent >= 256;
+    // (the persistent kernel does it always)
+    const bool rowpar = engine || max_col_ent >= 256;
+    const size_t o_kr = engine ? take(sizeof(c64) * W * max_col_ent) : 0;
     const size_t o_coefa = rowpar ? take(sizeof(c64) * 2 * W * n_z) : 0;
     const size_t o_coefb = rowpar ? take(sizeof(c64) * W * n_z) : 0;
     const size_t o_eta = rowpar ? take(sizeof(double) * W * n_z) : 0;
@@ -246,9 +287,9 @@ int run_solver(tb_ctx *ctx, const tb_bsr *H, const tb_bsr *S, const double *z, i
         if (has_s) {
             convert_values(opts.precision, (const double *)d_sval, sb + o_s32, S->nnzb * bb, stream);
             sval = sb + o_s32;
-            if (ir) convert_values(TB_PREC_MIXED, (const double *)d_sval, sb + o_sf32, S->nnzb * bb, stream);
         }
     }
+    if (ir) convert_values(TB_PREC_MIXED, (const double *)d_sval, sb + o_sf32, S->nnzb * bb, stream);
     TB_CUDA_TRY(ctx, cudaGetLastError());
 
     // ---- panel parameters
@@ -272,7 +313,11 @@ int run_solver(tb_ctx *ctx, const tb_bsr *H, const tb_bsr *S, const double *z, i
         p.P[0] = vec();
         p.P[1] = vec();
     }
-    if (has_s) {
+    if (engine) p.P[0] = vec();
+    if (engine && has_s) {
+        p.R[0] = vec();
+        p.Tv = vec();
+    } else if (has_s) {
         p.R[0] = vec();
         p.R[1] = vec();
         if (mixed)
@@ -320,16 +365,11 @@ int run_solver(tb_ctx *ctx, const tb_bsr *H, const tb_bsr *S, const double *z, i
     p.tol = opts.tol;
     // df64 restarts (see k_outer); not with gsQMR, whose smoothing runs over one seed's iterates
     p.stall2 = (opts.precision == TB_PREC_DF64 && !qmr) ? 1e-20 : 0.0;
-    // inner tolerance: FP64 and FP32 panels 1e-3 tol (floors 1e-13, 1e-7); df panels
-    // refine to 1e-5 tol (floor 1e-12): the refinement makes the tighter target cheap,
-    // and inexact inner solves are what separates the shifted results from the FP64 ones
-    p.inner_tol = opts.inner_tol > 0.0 ? opts.inner_tol
-                                       : (ir ? std::max(1e-5 * opts.tol, 1e-12)
-                                             : std::max(1e-3 * opts.tol, mixed ? 1e-7 : (lowp ? 1e-12 : 1e-13)));
+    p.inner_tol = inner_tol;
     p.refine_max = 8;
     p.sweep_red = 1e-5;
     p.max_iter = opts.max_iter;
-    p.inner_max = opts.inner_max > 0 ? opts.inner_max : 40;
+    p.inner_max = inner_max;
     // loop executions: while the queue is not empty every slot is busy, so at most
     // n_rhs (max_iter + 2) / W of them, then at most max_iter + 2 for the last columns
     p.outer_cap = (n_rhs * ((int64_t)opts.max_iter + 2) + W - 1) / W + opts.max_iter + 2;
@@ -339,6 +379,38 @@ int run_solver(tb_ctx *ctx, const tb_bsr *H, const tb_bsr *S, const double *z, i
     p.status = (int32_t *)d_status;
     p.stats = (int64_t *)(sb + o_stats);
 
+    if (engine) {
+        GridBarrier *bar = (GridBarrier *)(sb + o_bar);
+        TB_CUDA_TRY(ctx, cudaMemsetAsync(bar, 0, sizeof(GridBarrier), stream));
+        if (profiling) p.outer_cap = profile_reps;
+        en.p = p;
+        en.bar = bar;
+        en.sc = (SlotScalars<double> *)(sb + o_sc);
+        en.W = W;
+        en.kr = (c64 *)(sb + o_kr);
+        en.profile = profiling;
+        if (ir) en.X[0] = p.C32, en.X[1] = p.A32;
+        EngineLaunch E{ctx, en, has_s, opts.ctas_per_sm, num_sms(), stream};
+        if (!(lowp ? launch_engine_df(E, b) : launch_engine_f64(E, b)))
+            return set_error(ctx, TB_ERR_UNSUPPORTED, "no solver variant for b=%d", b);
+        if (E.rc) return E.rc;
+        GridBarrier hb;
+        TB_CUDA_TRY(ctx, cudaMemcpyAsync(&hb, bar, sizeof(hb), cudaMemcpyDeviceToHost, stream));
+        TB_CUDA_TRY(ctx, cudaStreamSynchronize(stream));
+        TB_CHECK(ctx, !hb.err, TB_ERR_CUDA, "panel solver: a grid barrier timed out");
+        if (hb.fail) // the bounds missed part of S's spectrum
+            return run_solver(ctx, H, S, z, n_z, rhs_rows, n_rhs, out_row_ptr, out_rows, &opts, G, iters, resid, status,
+                              profile_reps, ms, true);
+        if (profiling) {
+            const int ph[7] = {PH_A, PH_B, has_s ? PH_X : PH_INIT, PH_INIT, PH_INIT, PH_R, PH_R32};
+            double outer = 0;
+            for (int k = 0; k < 7; ++k)
+                ms[k] = ph[k] != PH_INIT && hb.cnt[ph[k]] ? 1e-6 * (double)hb.ns[ph[k]] / (double)hb.cnt[ph[k]] : 0.0;
+            for (int k = 0; k < 7; ++k) outer += 1e-6 * (double)hb.ns[k];
+            ms[7] = outer / std::max<double>(1, (double)hb.cnt[PH_A]);
+            return TB_OK;
+        }
+    } else {
     SolveLaunch L{ctx, has_s, ncta, n_rows, stream, profile_reps, ms};
     L.pd = p;
     L.ncta_a = ncta_a;
@@ -351,6 +423,7 @@ int run_solver(tb_ctx *ctx, const tb_bsr *H, const tb_bsr *S, const double *z, i
     if (L.rc) return L.rc;
     TB_CUDA_TRY(ctx, cudaGetLastError());
     if (profiling) return TB_OK;
+    }
     if (opts.stats) {
         TB_CUDA_TRY(ctx, cudaMemcpy(opts.stats, sb + o_stats, sizeof(int64_t) * 4, cudaMemcpyDeviceToHost));
     }
@@ -374,8 +447,7 @@ int run_solver(tb_ctx *ctx, const tb_bsr *H, const tb_bsr *S, const double *z, i
 int autotune(tb_ctx *ctx, const tb_bsr *H, const tb_bsr *S, const double *z, int32_t n_z, const int64_t *rhs_rows,
              int64_t n_rhs, const int64_t *out_row_ptr, const int64_t *out_rows, const tb_solve_opts &opts,
              int *W_out, int *cps_out) {
-    const bool mixed = opts.precision == TB_PREC_MIXED;
-    *W_out = panel_width_for((int)std::min<int64_t>(n_rhs, mixed ? 64 : 32));
+    *W_out = 0; // run_solver's own choice
     *cps_out = opts.ctas_per_sm;
     if (n_rhs < 128) return TB_OK; // tuning would cost more than it saves
     tb_tune_key key{H->n_brows, H->nnzb, std::min<int64_t>(n_rhs, 64), H->bdim, S ? 1 : 0, opts.precision, n_z};
@@ -400,7 +472,7 @@ int autotune(tb_ctx *ctx, const tb_bsr *H, const tb_bsr *S, const double *z, int
                                 nullptr, 2, ms);
             if (rc < 0) return rc;
             const double inner = S ? 8.0 : 0.0;
-            const double per_col = (ms[0] + ms[1] + ms[4] + inner * (ms[2] + ms[3])) / W;
+            const double per_col = (ms[7] > 0 ? ms[7] : ms[0] + ms[1] + ms[4] + inner * (ms[2] + ms[3])) / W;
             if (per_col < best) {
                 best = per_col;
                 *W_out = W;

@@ -12,6 +12,7 @@
 namespace tbgf {
 
 constexpr int NT = 256;
+constexpr int MAX_W = 64; // slots of a panel at most
 
 // ------------------------------------------------------------------ init
 // Column state of a slot that starts column `col` of the queue (or an empty,
@@ -61,8 +62,8 @@ __device__ __forceinline__ ShiftState fresh_shift() {
 // the queue) starts its recurrences again with beta = 0: what it keeps by
 // recurrence (u and p; FP32 panels: p and S p) is cleared, so that nothing of the old
 // column (not even an inf or a NaN) survives the multiplication by zero.
-template <typename T, int W>
-__device__ __forceinline__ void clear_restart_row(const Panel<T> &p, int n, int64_t row, int col) {
+template <typename T>
+__device__ __forceinline__ void clear_restart_row(const Panel<T> &p, int W, int n, int64_t row, int col) {
     const int64_t o = (row * W + col) * 2;
     T *pp = p.P[1] ? p.P[n & 1] : p.P[0]; // FP32 panels alternate between two buffers
     if (pp) pp[o] = pp[o + 1] = (T)0;
@@ -152,130 +153,170 @@ constexpr int ctas_light() {
 // the shift's COCG residual (rho_n = r_n^T S r_n), 1/tau_n^2 = 1/tau_{n-1}^2 +
 // 1/omega_n^2 and xq_n = xq_{n-1} + (tau_n^2 / omega_n^2)(x_n - xq_{n-1}); the shift
 // stops when tau_n / tau_0 <= tol.
+struct PairSmem {
+    c64 a[PAIR_CHUNK], b[PAIR_CHUNK];
+    double eta[PAIR_CHUNK];
+    int c[PAIR_CHUNK], m[PAIR_CHUNK], on[PAIR_CHUNK];
+};
+
+// This CTA's range of the W * nz (slot, shift) pairs.
+template <typename T>
+__device__ __forceinline__ void pair_range(const Panel<T> &p, int W, int &q0, int &q1) {
+    const int64_t P = (int64_t)W * p.nz;
+    q0 = (int)((int64_t)blockIdx.x * P / gridDim.x), q1 = (int)((int64_t)(blockIdx.x + 1) * P / gridDim.x);
+}
+
+// Phase 1 of A for pair q: recurrence, residual test, coefficients.
+struct PairA {
+    int on;     // bit 0: p^m update with a, b; bit 1: smoothing update with eta
+    c64 a, b;
+    double eta;
+};
+template <typename T>
+__device__ __forceinline__ PairA pair_coef_A(const Panel<T> &p, int q, int n) {
+    PairA r;
+    r.on = 0;
+    r.a = r.b = mk(0.0, 0.0);
+    r.eta = 0.0;
+    ColState &C = p.col[q / p.nz];
+    ShiftState &S = p.sh[q];
+    if (C.done || !S.active) return r;
+    S.pi_prev = S.pi;
+    S.pi = S.pi_next;
+    double res;
+    if (p.qmr) {
+        const double w2inv = cabs2(S.pi) / sqrt(cabs2(C.rho)); // 1 / omega_n^2
+        if (S.qinv == 0.0) S.qinv0 = w2inv;
+        S.qinv += w2inv;
+        r.eta = w2inv / S.qinv;
+        res = sqrt(S.qinv0 / S.qinv);
+        r.on = 2; // smoothing update of the kept rows
+    } else {
+        res = sqrt(C.rn2) / sqrt(cabs2(S.pi));
+    }
+    S.resid = res;
+    if (res <= p.tol) {
+        S.active = 0;
+        S.conv_it = n;
+        atomicSub(&C.n_active, 1);
+    } else {
+        const c64 ratio = cdiv(S.pi_prev, S.pi);
+        r.b = (ratio * ratio) * C.beta_prev;
+        r.a = cdiv(mk(1.0, 0.0), S.pi);
+        r.on |= 1;
+    }
+    return r;
+}
+// ... left for the row-parallel updates
+template <typename T>
+__device__ __forceinline__ void pair_store_A(const Panel<T> &p, int q, const PairA &r) {
+    p.flagA[q] = r.on;
+    if (r.on & 1) p.coefA[2 * q] = r.a, p.coefA[2 * q + 1] = r.b;
+    if (r.on & 2) p.etaA[q] = r.eta;
+}
+
+// Phase 2 of A for np pairs: p^m (and the QMR iterate) on the kept rows.  W: the panel's row stride.
+template <typename T>
+__device__ __forceinline__ void pair_rows_A(const Panel<T> &p, const PairSmem &s, int np, int W, const T *Rc) {
+    const int KM = p.max_col_ent;
+    // pairs fastest: the pairs of a chunk are consecutive shifts of a column, so
+    // consecutive threads touch consecutive entries of a kept row (coalesced)
+    for (int64_t i = threadIdx.x; i < (int64_t)np * KM; i += blockDim.x) {
+        const int t = (int)(i % np), k = (int)(i / np);
+        if (!s.on[t]) continue;
+        const int c = s.c[t], m = s.m[t];
+        const ColState &C = p.col[c];
+        if (k >= C.n_ent) continue;
+        const int64_t e = ((int64_t)c * KM + k) * p.nz + m;
+        if (s.on[t] & 2) p.xq[e] = p.xq[e] + s.eta[t] * (p.xs[e] - p.xq[e]);
+        if (!(s.on[t] & 1)) continue;
+        const int64_t row = p.ent_row[C.ent0 + k];
+        const T *rp = Rc + (row * W + c) * 2;
+        const c64 rv = mk((double)rp[0], (double)rp[1]);
+        p.ps[e] = s.a[t] * rv + s.b[t] * p.ps[e];
+    }
+}
+
 template <typename T, int W>
 __device__ void pair_step_A(const Panel<T> &p, const T *__restrict__ Rc, int n) {
-    __shared__ c64 s_a[PAIR_CHUNK], s_b[PAIR_CHUNK];
-    __shared__ double s_eta[PAIR_CHUNK];
-    __shared__ int s_c[PAIR_CHUNK], s_m[PAIR_CHUNK], s_on[PAIR_CHUNK];
-    const int P = W * p.nz;
-    const int q0 = (int)((int64_t)blockIdx.x * P / gridDim.x), q1 = (int)((int64_t)(blockIdx.x + 1) * P / gridDim.x);
-    const int KM = p.max_col_ent;
+    __shared__ PairSmem s;
+    int q0, q1;
+    pair_range(p, W, q0, q1);
     for (int base = q0; base < q1; base += PAIR_CHUNK) {
         const int np = min(PAIR_CHUNK, q1 - base);
         for (int t = threadIdx.x; t < np; t += blockDim.x) {
-            const int q = base + t, c = q / p.nz, m = q % p.nz;
-            int on = 0;
-            ColState &C = p.col[c];
-            ShiftState &S = p.sh[q];
-            if (!C.done && S.active) {
-                S.pi_prev = S.pi;
-                S.pi = S.pi_next;
-                double res;
-                if (p.qmr) {
-                    const double w2inv = cabs2(S.pi) / sqrt(cabs2(C.rho)); // 1 / omega_n^2
-                    if (S.qinv == 0.0) S.qinv0 = w2inv;
-                    S.qinv += w2inv;
-                    s_eta[t] = w2inv / S.qinv;
-                    res = sqrt(S.qinv0 / S.qinv);
-                    on = 2; // smoothing update of the kept rows
-                } else {
-                    res = sqrt(C.rn2) / sqrt(cabs2(S.pi));
-                }
-                S.resid = res;
-                if (res <= p.tol) {
-                    S.active = 0;
-                    S.conv_it = n;
-                    atomicSub(&C.n_active, 1);
-                } else {
-                    const c64 ratio = cdiv(S.pi_prev, S.pi);
-                    s_b[t] = (ratio * ratio) * C.beta_prev;
-                    s_a[t] = cdiv(mk(1.0, 0.0), S.pi);
-                    on |= 1;
-                }
-            }
-            s_on[t] = on;
-            s_c[t] = c;
-            s_m[t] = m;
-            if (p.rowpar) { // k_rows_A applies them
-                p.flagA[q] = on;
-                if (on & 1) p.coefA[2 * q] = s_a[t], p.coefA[2 * q + 1] = s_b[t];
-                if (on & 2) p.etaA[q] = s_eta[t];
-            }
+            const PairA r = pair_coef_A(p, base + t, n);
+            s.on[t] = r.on, s.a[t] = r.a, s.b[t] = r.b, s.eta[t] = r.eta;
+            s.c[t] = (base + t) / p.nz, s.m[t] = (base + t) % p.nz;
+            if (p.rowpar) pair_store_A(p, base + t, r);
         }
         __syncthreads();
         if (p.rowpar) continue;
-        // pairs fastest: the pairs of a chunk are consecutive shifts of a column, so
-        // consecutive threads touch consecutive entries of a kept row (coalesced)
-        for (int64_t i = threadIdx.x; i < (int64_t)np * KM; i += blockDim.x) {
-            const int t = (int)(i % np), k = (int)(i / np);
-            if (!s_on[t]) continue;
-            const int c = s_c[t], m = s_m[t];
-            const ColState &C = p.col[c];
-            if (k >= C.n_ent) continue;
-            const int64_t e = ((int64_t)c * KM + k) * p.nz + m;
-            if (s_on[t] & 2) p.xq[e] = p.xq[e] + s_eta[t] * (p.xs[e] - p.xq[e]);
-            if (!(s_on[t] & 1)) continue;
-            const int64_t row = p.ent_row[C.ent0 + k];
-            const T *rp = Rc + (row * W + c) * 2;
-            const c64 rv = mk((double)rp[0], (double)rp[1]);
-            p.ps[e] = s_a[t] * rv + s_b[t] * p.ps[e];
-        }
+        pair_rows_A(p, s, np, W, Rc);
         __syncthreads();
     }
 }
 
 // B(n) / B'(n): pi_{n+1}, alpha^m_n and x^m += alpha^m_n p^m_n on the kept rows.
+// Phase 1 of B for pair q: pi_{n+1} and as = alpha^m_n; false: no update.
+template <typename T>
+__device__ __forceinline__ bool pair_coef_B(const Panel<T> &p, int q, c64 &as) {
+    as = mk(0.0, 0.0);
+    ColState &C = p.col[q / p.nz];
+    ShiftState &S = p.sh[q];
+    if (C.done || !S.active) return false;
+    const c64 sig = p.z[q % p.nz] - C.zs;
+    const c64 coef = cdiv(C.alpha * C.beta_prev, C.alpha_prev);
+    const c64 pn = (mk(1.0, 0.0) + C.alpha * sig) * S.pi + coef * (S.pi - S.pi_prev);
+    as = cdiv(S.pi, pn) * C.alpha;
+    if (!cfinite(pn) || (pn.re == 0.0 && pn.im == 0.0) || !cfinite(as)) {
+        S.active = 0;
+        S.resid = nan("");
+        C.breakdown = 1;
+        atomicSub(&C.n_active, 1);
+        return false;
+    }
+    S.pi_next = pn;
+    S.alpha_s = as;
+    return true;
+}
+template <typename T>
+__device__ __forceinline__ void pair_store_B(const Panel<T> &p, int q, bool on, c64 as) {
+    p.flagB[q] = on;
+    if (on) p.coefB[q] = as;
+}
+
+// Phase 2 of B for np pairs: x^m on the kept rows (pairs fastest, as in A).
+template <typename T>
+__device__ __forceinline__ void pair_rows_B(const Panel<T> &p, const PairSmem &s, int np) {
+    const int KM = p.max_col_ent;
+    for (int64_t i = threadIdx.x; i < (int64_t)np * KM; i += blockDim.x) {
+        const int t = (int)(i % np), k = (int)(i / np);
+        if (!s.on[t]) continue;
+        const int c = s.c[t], m = s.m[t];
+        if (k >= p.col[c].n_ent) continue;
+        const int64_t e = ((int64_t)c * KM + k) * p.nz + m;
+        p.xs[e] = p.xs[e] + s.a[t] * p.ps[e];
+    }
+}
+
 template <typename T, int W>
 __device__ void pair_step_B(const Panel<T> &p) {
-    __shared__ c64 s_a[PAIR_CHUNK];
-    __shared__ int s_c[PAIR_CHUNK], s_m[PAIR_CHUNK], s_on[PAIR_CHUNK];
-    const int P = W * p.nz;
-    const int q0 = (int)((int64_t)blockIdx.x * P / gridDim.x), q1 = (int)((int64_t)(blockIdx.x + 1) * P / gridDim.x);
-    const int KM = p.max_col_ent;
+    __shared__ PairSmem s;
+    int q0, q1;
+    pair_range(p, W, q0, q1);
     for (int base = q0; base < q1; base += PAIR_CHUNK) {
         const int np = min(PAIR_CHUNK, q1 - base);
         for (int t = threadIdx.x; t < np; t += blockDim.x) {
-            const int q = base + t, c = q / p.nz, m = q % p.nz;
-            int on = 0;
-            ColState &C = p.col[c];
-            ShiftState &S = p.sh[q];
-            if (!C.done && S.active) {
-                const c64 sig = p.z[m] - C.zs;
-                const c64 coef = cdiv(C.alpha * C.beta_prev, C.alpha_prev);
-                const c64 pn = (mk(1.0, 0.0) + C.alpha * sig) * S.pi + coef * (S.pi - S.pi_prev);
-                const c64 as = cdiv(S.pi, pn) * C.alpha;
-                if (!cfinite(pn) || (pn.re == 0.0 && pn.im == 0.0) || !cfinite(as)) {
-                    S.active = 0;
-                    S.resid = nan("");
-                    C.breakdown = 1;
-                    atomicSub(&C.n_active, 1);
-                } else {
-                    S.pi_next = pn;
-                    S.alpha_s = as;
-                    s_a[t] = as;
-                    on = 1;
-                }
-            }
-            s_on[t] = on;
-            s_c[t] = c;
-            s_m[t] = m;
-            if (p.rowpar) { // k_rows_B applies it
-                p.flagB[q] = on;
-                if (on) p.coefB[q] = s_a[t];
-            }
+            c64 as;
+            const bool on = pair_coef_B(p, base + t, as);
+            s.on[t] = on, s.a[t] = as;
+            s.c[t] = (base + t) / p.nz, s.m[t] = (base + t) % p.nz;
+            if (p.rowpar) pair_store_B(p, base + t, on, as);
         }
         __syncthreads();
         if (p.rowpar) continue;
-        // pairs fastest: the pairs of a chunk are consecutive shifts of a column, so
-        // consecutive threads touch consecutive entries of a kept row (coalesced)
-        for (int64_t i = threadIdx.x; i < (int64_t)np * KM; i += blockDim.x) {
-            const int t = (int)(i % np), k = (int)(i / np);
-            if (!s_on[t]) continue;
-            const int c = s_c[t], m = s_m[t];
-            if (k >= p.col[c].n_ent) continue;
-            const int64_t e = ((int64_t)c * KM + k) * p.nz + m;
-            p.xs[e] = p.xs[e] + s_a[t] * p.ps[e];
-        }
+        pair_rows_B(p, s, np);
         __syncthreads();
     }
 }
@@ -303,8 +344,7 @@ __device__ __forceinline__ void rows_index(int64_t t, int64_t per, int nz, bool 
 
 template <typename T, int W>
 __global__ void k_rows_A(Panel<T> p, int has_s) {
-    const int n = p.ctl->n;
-    const T *Rc = has_s ? p.R[n & 1] : p.RT;
+    const T *Rc = has_s ? p.R[p.ctl->n & 1] : p.RT;
     const int64_t KM = p.max_col_ent, per = KM * p.nz;
     const bool small = W * per < (int64_t)UINT32_MAX;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -342,18 +382,173 @@ __global__ void k_rows_B(Panel<T> p) {
     }
 }
 
+
+// End of A (last CTA): alpha_n = rho_n / mu_n from red[2 c], red[2 c + 1] = mu_n of
+// slot c, on the column states col (p.col, or the caller's copy); column completion,
+// retire, refill and restart.  Returns (in every thread) whether some slot's column
+// finished.
+template <typename T>
+__device__ bool finish_alpha(const Panel<T> &p, int W, const double *red, ColState *col) {
+    __shared__ int fin[MAX_W], n_fin; // slots whose column finished in this iteration
+    if (threadIdx.x == 0) n_fin = 0;
+    __syncthreads();
+    // (everything a slot's decision needs is loaded before the first branch: the last
+    // CTA works alone, and each dependent L2 trip costs it a third of a microsecond)
+    for (int c = threadIdx.x; c < W; c += NT) {
+        ColState &C = col[c];
+        const int done = C.done, s_bad = C.s_bad, breakdown = C.breakdown, its = C.iters;
+        const int n_active = C.n_active;
+        const c64 rho = C.rho;
+        if (done) continue;
+        const c64 mu = mk(red[2 * c], red[2 * c + 1]);
+        int st = -1;
+        if (s_bad)
+            st = TB_COL_BREAKDOWN; // S is not positive definite on an inner CG direction
+        else if (n_active <= 0)
+            st = breakdown ? TB_COL_BREAKDOWN : TB_COL_CONVERGED;
+        else if (!cfinite(mu) || !cfinite(rho))
+            st = TB_COL_NONFINITE;
+        else if ((mu.re == 0.0 && mu.im == 0.0) || (rho.re == 0.0 && rho.im == 0.0))
+            st = TB_COL_BREAKDOWN;
+        else if (its >= p.max_iter)
+            st = TB_COL_MAX_ITER;
+        c64 a = mk(0.0, 0.0);
+        if (st < 0) {
+            a = cdiv(rho, mu);
+            if (!cfinite(a)) st = TB_COL_NONFINITE;
+        }
+        if (st >= 0) {
+            C.done = 1;
+            C.status = st;
+            C.alpha = mk(0.0, 0.0);
+            fin[atomicAdd(&n_fin, 1)] = c;
+        } else {
+            C.alpha = a;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) // slots take the queue's columns in slot order (deterministic)
+        for (int f = 1; f < n_fin; ++f)
+            for (int g = f; g > 0 && fin[g - 1] > fin[g]; --g) {
+                const int x = fin[g];
+                fin[g] = fin[g - 1];
+                fin[g - 1] = x;
+            }
+    __syncthreads();
+    if (n_fin > 0) {
+        // retire: the finished columns' results go out now, so that their slots
+        // can take the next columns of the queue in this same iteration
+        const int KM = p.max_col_ent;
+        for (int f = 0; f < n_fin; ++f) {
+            const ColState &C = col[fin[f]];
+            const int64_t base = (int64_t)fin[f] * KM * p.nz, ne = (int64_t)C.n_ent * p.nz;
+            const c64 *xo = p.qmr ? p.xq : p.xs;
+            if (!p.G) continue; // profiling: no outputs
+            for (int64_t t = threadIdx.x; t < ne; t += NT) {
+                c64 v = xo[base + t];
+                if (p.rowpar && p.qmr) { // this iteration's smoothing step is still pending (k_rows_A)
+                    const int64_t q = (int64_t)fin[f] * p.nz + t % p.nz;
+                    if (p.flagA[q] & 2) v = v + p.etaA[q] * (p.xs[base + t] - v);
+                }
+                p.G[C.ent0 * p.nz + t] = v;
+            }
+            for (int m = threadIdx.x; m < p.nz; m += NT)
+                p.resid[C.dst * p.nz + m] = p.sh[(int64_t)fin[f] * p.nz + m].resid;
+        }
+        __syncthreads();
+        // refill: the next column starts through the restart path (alpha = 0 this
+        // iteration, B / B' set its rt to e_j and clear its old directions, C
+        // starts its recurrences); the restart iteration is not counted
+        for (int f = threadIdx.x; f < n_fin; f += NT) {
+            ColState &C = col[fin[f]];
+            if (p.G) {
+                p.iters[C.dst] = C.iters;
+                p.status[C.dst] = C.status;
+            }
+            const int64_t next = (int64_t)atomicAdd(reinterpret_cast<unsigned long long *>(&p.ctl->next_col), 1ull);
+            ColState N = fresh_column(p, next);
+            if (N.dst >= 0) {
+                N.restart = 1;
+                N.fresh = 1;
+                N.iters = -1;
+            }
+            C = N;
+        }
+        __syncthreads();
+        for (int f = 0; f < n_fin; ++f) {
+            const int c = fin[f];
+            if (col[c].dst < 0) continue; // the queue is empty: the slot stays idle
+            for (int m = threadIdx.x; m < p.nz; m += NT) p.sh[(int64_t)c * p.nz + m] = fresh_shift();
+            const int64_t base = (int64_t)c * KM * p.nz;
+            for (int64_t t = threadIdx.x; t < (int64_t)KM * p.nz; t += NT) {
+                p.xs[base + t] = mk(0.0, 0.0);
+                p.ps[base + t] = mk(0.0, 0.0);
+                if (p.xq) p.xq[base + t] = mk(0.0, 0.0);
+            }
+        }
+        __syncthreads();
+    }
+    // Restart (df panels): a shift's residual is the seed's divided by |pi|, so
+    // a shift much harder than the seed needs the seed residual below what df
+    // carries (about 1e-10).  Once a column's seed residual is below that, its
+    // worst active shift is checked every 512 iterations; if it improved by
+    // less than 1 % the column restarts with that shift as its seed: alpha = 0
+    // this iteration, B / B' reset rt to e_j, C restarts the recurrences;
+    // converged shifts keep their solutions, active ones start from zero.
+    if (p.stall2 > 0.0) {
+        const int KM = p.max_col_ent;
+        for (int c = threadIdx.x; c < W; c += NT) {
+            ColState &C = col[c];
+            const double rn2 = C.rn2;
+            const int done = C.done, restarts = C.restarts, chk = C.chk_n, its = C.iters;
+            if (done || !(rn2 < p.stall2) || restarts >= 2) continue;
+            if (chk >= 0 && its - chk < 512) continue;
+            double rw = -1.0;
+            int mw = -1;
+            for (int m = 0; m < p.nz; ++m) {
+                const ShiftState &S = p.sh[(int64_t)c * p.nz + m];
+                if (S.active && S.resid > rw) rw = S.resid, mw = m;
+            }
+            if (mw < 0) continue;
+            if (C.chk_n < 0 || rw < 0.99 * C.chk_w) {
+                C.chk_n = C.iters;
+                C.chk_w = rw;
+                continue;
+            }
+            C.zs = p.z[mw];
+            C.restart = 1;
+            C.restarts += 1;
+            C.chk_n = -1;
+            C.alpha = mk(0.0, 0.0);
+            for (int m = 0; m < p.nz; ++m) {
+                ShiftState &S = p.sh[(int64_t)c * p.nz + m];
+                if (!S.active) continue;
+                S.pi = S.pi_prev = S.pi_next = mk(1.0, 0.0);
+                S.resid = 1.0;
+                for (int k = 0; k < C.n_ent; ++k) {
+                    p.xs[((int64_t)c * KM + k) * p.nz + m] = mk(0.0, 0.0);
+                    p.ps[((int64_t)c * KM + k) * p.nz + m] = mk(0.0, 0.0);
+                }
+            }
+        }
+    }
+    __syncthreads();
+    const int all = __syncthreads_and(threadIdx.x < W ? col[threadIdx.x].done != 0 : 1);
+    if (threadIdx.x == 0) p.ctl->panel_done = all;
+    return n_fin > 0;
+}
+
 // -------------------------------------------------------------- kernel A
 template <typename T, int B, int W, bool HAS_S>
 __global__ void __launch_bounds__(NT, (B <= 4 ? 3 : 1)) k_outer(Panel<T> p) {
     using TM = Teams<T, W, NT>;
     constexpr int CPT = TM::CPT;
     const int team = threadIdx.x / TM::TPR, lane = threadIdx.x % TM::TPR;
-    // FP64 and df panels keep u = (z_s S - H) p_n by recurrence, u_n = z_s rt_n -
-    // H r_n + beta u_{n-1}, so no S p or H p is stored and the product reads
-    // finished rows.  S = I: mu_n = p_n^T u_n = r_n^T u_n (p_{n-1}^T u_n = 0), no p
-    // either: r and u in, u out, 3 panel vectors instead of 6.  With S, r = S^-1 rt
-    // carries the inner solve's error, with which r^T u costs up to 30 % more
-    // iterations (the p^T u form 4 %), so p is kept: 6 vectors instead of 9.
+    // FP64 and df panels (S != I here) keep u = (z_s S - H) p_n by recurrence, u_n = z_s
+    // rt_n - H r_n + beta u_{n-1}, so no S p or H p is stored and the product reads
+    // finished rows: 6 panel vectors instead of 9.  (mu_n = r_n^T u_n, which is p_n^T u_n
+    // in exact arithmetic, would save p too, but takes up to 30 % more iterations with
+    // the inner solve's error in r, and some columns 20 % more without S.)
     // FP32 panels form p_n on the fly and multiply it.
     constexpr bool U_REC = !std::is_same<T, float>::value;
     const int n = p.ctl->n;
@@ -380,22 +575,17 @@ __global__ void __launch_bounds__(NT, (B <= 4 ? 3 : 1)) k_outer(Panel<T> p) {
 #pragma unroll
         for (int i = 0; i < B; ++i) {
             const int64_t row = br * B + i;
-            cpx<T> pv[CPT], u[CPT]; // p_n (r_n when S = I); u_n
+            cpx<T> pv[CPT], u[CPT]; // p_n; u_n
             ld(row, pv);
             if constexpr (U_REC) {
                 cpx<T> rt[CPT];
                 ld_row<T, W>(p.U, row, lane, u);
-                if constexpr (HAS_S) {
-                    cpx<T> po[CPT];
-                    ld_row<T, W>(p.P[0], row, lane, po);
-                    ld_row<T, W>(p.RT, row, lane, rt);
+                cpx<T> po[CPT];
+                ld_row<T, W>(p.P[0], row, lane, po);
+                ld_row<T, W>(p.RT, row, lane, rt);
 #pragma unroll
-                    for (int cc = 0; cc < CPT; ++cc) pv[cc] = pv[cc] + ld.s[cc] * po[cc];
-                    st_row<T, W>(p.P[0], row, lane, pv);
-                } else {
-#pragma unroll
-                    for (int cc = 0; cc < CPT; ++cc) rt[cc] = pv[cc];
-                }
+                for (int cc = 0; cc < CPT; ++cc) pv[cc] = pv[cc] + ld.s[cc] * po[cc];
+                st_row<T, W>(p.P[0], row, lane, pv);
 #pragma unroll
                 for (int cc = 0; cc < CPT; ++cc) u[cc] = (zs[cc] * rt[cc] - y[i][cc]) + ld.s[cc] * u[cc];
             } else {
@@ -428,174 +618,37 @@ __global__ void __launch_bounds__(NT, (B <= 4 ? 3 : 1)) k_outer(Panel<T> p) {
     cta_partials<T, W, NT, 2>(acc, p.part);
     pair_step_A<T, W>(p, Rc, n);
     if (!last_cta_arrival(&p.ctl->arrive)) return;
-    // ---- last CTA: alpha_n = rho_n / mu_n; column completion, retire and refill
     __shared__ double red[W * 2];
-    __shared__ int fin[W], n_fin; // slots whose column finished in this iteration
-    if (threadIdx.x == 0) n_fin = 0;
     reduce_partials<T, W, NT, 2>(p.part, red);
-    for (int c = threadIdx.x; c < W; c += NT) {
-        ColState &C = p.col[c];
-        if (C.done) continue;
-        const c64 mu = mk(red[2 * c], red[2 * c + 1]);
-        const int n_active = atomicAdd(&C.n_active, 0);
-        int st = -1;
-        if (C.s_bad)
-            st = TB_COL_BREAKDOWN; // S is not positive definite on an inner CG direction
-        else if (n_active <= 0)
-            st = C.breakdown ? TB_COL_BREAKDOWN : TB_COL_CONVERGED;
-        else if (!cfinite(mu) || !cfinite(C.rho))
-            st = TB_COL_NONFINITE;
-        else if ((mu.re == 0.0 && mu.im == 0.0) || (C.rho.re == 0.0 && C.rho.im == 0.0))
-            st = TB_COL_BREAKDOWN;
-        else if (C.iters >= p.max_iter)
-            st = TB_COL_MAX_ITER;
-        c64 a = mk(0.0, 0.0);
-        if (st < 0) {
-            a = cdiv(C.rho, mu);
-            if (!cfinite(a)) st = TB_COL_NONFINITE;
-        }
-        if (st >= 0) {
-            C.done = 1;
-            C.status = st;
-            C.alpha = mk(0.0, 0.0);
-            fin[atomicAdd(&n_fin, 1)] = c;
-        } else {
-            C.alpha = a;
-        }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) // slots take the queue's columns in slot order (deterministic)
-        for (int f = 1; f < n_fin; ++f)
-            for (int g = f; g > 0 && fin[g - 1] > fin[g]; --g) {
-                const int x = fin[g];
-                fin[g] = fin[g - 1];
-                fin[g - 1] = x;
-            }
-    __syncthreads();
-    if (n_fin > 0) {
-        // retire: the finished columns' results go out now, so that their slots
-        // can take the next columns of the queue in this same iteration
-        const int KM = p.max_col_ent;
-        for (int f = 0; f < n_fin; ++f) {
-            const ColState &C = p.col[fin[f]];
-            const int64_t base = (int64_t)fin[f] * KM * p.nz, ne = (int64_t)C.n_ent * p.nz;
-            const c64 *xo = p.qmr ? p.xq : p.xs;
-            for (int64_t t = threadIdx.x; t < ne; t += NT) {
-                c64 v = xo[base + t];
-                if (p.rowpar && p.qmr) { // this iteration's smoothing step is still pending (k_rows_A)
-                    const int64_t q = (int64_t)fin[f] * p.nz + t % p.nz;
-                    if (p.flagA[q] & 2) v = v + p.etaA[q] * (p.xs[base + t] - v);
-                }
-                p.G[C.ent0 * p.nz + t] = v;
-            }
-            for (int m = threadIdx.x; m < p.nz; m += NT)
-                p.resid[C.dst * p.nz + m] = p.sh[(int64_t)fin[f] * p.nz + m].resid;
-        }
-        __syncthreads();
-        // refill: the next column starts through the restart path (alpha = 0 this
-        // iteration, B / B' set its rt to e_j and clear its old directions, C
-        // starts its recurrences); the restart iteration is not counted
-        for (int f = threadIdx.x; f < n_fin; f += NT) {
-            ColState &C = p.col[fin[f]];
-            p.iters[C.dst] = C.iters;
-            p.status[C.dst] = C.status;
-            const int64_t next = (int64_t)atomicAdd(reinterpret_cast<unsigned long long *>(&p.ctl->next_col), 1ull);
-            ColState N = fresh_column(p, next);
-            if (N.dst >= 0) {
-                N.restart = 1;
-                N.fresh = 1;
-                N.iters = -1;
-            }
-            C = N;
-        }
-        __syncthreads();
-        for (int f = 0; f < n_fin; ++f) {
-            const int c = fin[f];
-            if (p.col[c].dst < 0) continue; // the queue is empty: the slot stays idle
-            for (int m = threadIdx.x; m < p.nz; m += NT) p.sh[(int64_t)c * p.nz + m] = fresh_shift();
-            const int64_t base = (int64_t)c * KM * p.nz;
-            for (int64_t t = threadIdx.x; t < (int64_t)KM * p.nz; t += NT) {
-                p.xs[base + t] = mk(0.0, 0.0);
-                p.ps[base + t] = mk(0.0, 0.0);
-                if (p.xq) p.xq[base + t] = mk(0.0, 0.0);
-            }
-        }
-        __syncthreads();
-    }
-    // Restart (df panels): a shift's residual is the seed's divided by |pi|, so
-    // a shift much harder than the seed needs the seed residual below what df
-    // carries (about 1e-10).  Once a column's seed residual is below that, its
-    // worst active shift is checked every 512 iterations; if it improved by
-    // less than 1 % the column restarts with that shift as its seed: alpha = 0
-    // this iteration, B / B' reset rt to e_j, C restarts the recurrences;
-    // converged shifts keep their solutions, active ones start from zero.
-    if (p.stall2 > 0.0) {
-        const int KM = p.max_col_ent;
-        for (int c = threadIdx.x; c < W; c += NT) {
-            ColState &C = p.col[c];
-            if (C.done || !(C.rn2 < p.stall2) || C.restarts >= 2) continue;
-            if (C.chk_n >= 0 && C.iters - C.chk_n < 512) continue;
-            double rw = -1.0;
-            int mw = -1;
-            for (int m = 0; m < p.nz; ++m) {
-                const ShiftState &S = p.sh[(int64_t)c * p.nz + m];
-                if (S.active && S.resid > rw) rw = S.resid, mw = m;
-            }
-            if (mw < 0) continue;
-            if (C.chk_n < 0 || rw < 0.99 * C.chk_w) {
-                C.chk_n = C.iters;
-                C.chk_w = rw;
-                continue;
-            }
-            C.zs = p.z[mw];
-            C.restart = 1;
-            C.restarts += 1;
-            C.chk_n = -1;
-            C.alpha = mk(0.0, 0.0);
-            for (int m = 0; m < p.nz; ++m) {
-                ShiftState &S = p.sh[(int64_t)c * p.nz + m];
-                if (!S.active) continue;
-                S.pi = S.pi_prev = S.pi_next = mk(1.0, 0.0);
-                S.resid = 1.0;
-                for (int k = 0; k < C.n_ent; ++k) {
-                    p.xs[((int64_t)c * KM + k) * p.nz + m] = mk(0.0, 0.0);
-                    p.ps[((int64_t)c * KM + k) * p.nz + m] = mk(0.0, 0.0);
-                }
-            }
-        }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int all = 1;
-        for (int c = 0; c < W; ++c) all &= (p.col[c].done != 0);
-        p.ctl->panel_done = all;
-    }
+    finish_alpha(p, W, red, p.col);
 }
 
 // Common end of an outer iteration (last CTA): beta_n, rotation, loop condition.
-template <typename T, int W>
-__device__ void finish_outer(const Panel<T> &p, const double *rho_next, int init) {
+template <typename T>
+__device__ void finish_outer(const Panel<T> &p, int W, const double *rho_next, int init, ColState *col) {
     for (int c = threadIdx.x; c < W; c += NT) {
-        ColState &C = p.col[c];
-        if (C.done) continue;
+        ColState &C = col[c];
+        const int done = C.done, restart = C.restart, its = C.iters;
+        const c64 rho = C.rho, alpha = C.alpha;
+        if (done) continue;
         const c64 rn = mk(rho_next[2 * c], rho_next[2 * c + 1]);
         if (init) {
             C.rho = rn;
             continue;
         }
-        if (C.restart) { // first iteration of the new seed follows
+        if (restart) { // first iteration of the new seed follows
             C.beta_prev = mk(0.0, 0.0);
             C.alpha_prev = mk(1.0, 0.0);
             C.rho = rn;
             C.restart = 0;
             C.fresh = 0;
-            C.iters += 1;
+            C.iters = its + 1;
             continue;
         }
-        C.beta_prev = cdiv(rn, C.rho);
-        C.alpha_prev = C.alpha;
+        C.beta_prev = cdiv(rn, rho);
+        C.alpha_prev = alpha;
         C.rho = rn;
-        C.iters += 1;
+        C.iters = its + 1;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -639,7 +692,7 @@ __global__ void __launch_bounds__(NT, (B <= 4 ? 3 : 1)) k_update_sI(Panel<T> p) 
             for (int cc = 0; cc < CPT; ++cc) {
                 if (rst >> cc & 1u) {
                     rt[cc] = mk<T>(row == p.col[lane * CPT + cc].row ? (T)1 : (T)0, 0);
-                    clear_restart_row<T, W>(p, p.ctl->n, row, lane * CPT + cc);
+                    clear_restart_row(p, W, p.ctl->n, row, lane * CPT + cc);
                 } else {
                     rt[cc] = rt[cc] - a[cc] * u[cc];
                 }
@@ -665,7 +718,7 @@ __global__ void __launch_bounds__(NT, (B <= 4 ? 3 : 1)) k_update_sI(Panel<T> p) 
         if (!p.col[c].done) p.col[c].rn2 = red[3 * c + 2];
     }
     __syncthreads();
-    finish_outer<T, W>(p, rho_next, 0);
+    finish_outer(p, W, rho_next, 0, p.col);
 }
 
 // -------------------------------------------------------------- kernel B' (S != I)
@@ -718,7 +771,7 @@ __global__ void __launch_bounds__(NT, (B <= 4 ? 3 : 1)) k_update_S(Panel<T> p) {
                 y0[cc] = mk((T)g[cc].re, (T)g[cc].im);
                 if (rst >> cc & 1u) {
                     rt[cc] = mk<T>(row == p.col[lane * CPT + cc].row ? (T)1 : (T)0, 0);
-                    clear_restart_row<T, W>(p, n, row, lane * CPT + cc);
+                    clear_restart_row(p, W, n, row, lane * CPT + cc);
                 } else {
                     rt[cc] = rt[cc] - a[cc] * u[cc];
                 }
@@ -1098,7 +1151,7 @@ __global__ void __launch_bounds__(NT, ctas_light<T, B>()) k_rho(Panel<T> p, int 
     if (!last_cta_arrival(&p.ctl->arrive)) return;
     __shared__ double red[W * 2];
     reduce_partials<T, W, NT, 2>(p.part, red);
-    finish_outer<T, W>(p, red, init);
+    finish_outer(p, W, red, init, p.col);
 }
 
 // -------------------------------------------------------------- write-out
@@ -1278,13 +1331,13 @@ struct SolveLaunch {
             cudaEventRecord(ev[0], stream);
             if (has_s)
                 k_outer<T, B, W, true><<<grid, block, 0, stream>>>(p);
-            else
+            else if constexpr (std::is_same<T, float>::value)
                 k_outer<T, B, W, false><<<grid, block, 0, stream>>>(p);
             if (p.rowpar) k_rows_A<T, W><<<rows_grid(p, W), block, 0, stream>>>(p, has_s_i);
             cudaEventRecord(ev[1], stream);
             if (has_s)
                 k_update_S<T, B, W><<<grid, block, 0, stream>>>(p);
-            else
+            else if constexpr (std::is_same<T, float>::value)
                 k_update_sI<T, B, W><<<grid, block, 0, stream>>>(p);
             if (p.rowpar) k_rows_B<T, W><<<rows_grid(p, W), block, 0, stream>>>(p);
             cudaEventRecord(ev[2], stream);
@@ -1402,7 +1455,7 @@ struct SolveLaunch {
                 x = gb.add_while(ob, p_body.h_inner, &x, 1, &ib);
                 if (!gb.rc) inner_body(ib, a_body, a_fbody);
                 gb.add_kernel(ob, (const void *)k_rho<T, B, W>, grid_a, block, a_body_rho, &x, 1);
-            } else {
+            } else if constexpr (std::is_same<T, float>::value) { // (FP64 and df panels without S: engine.cuh)
                 cudaGraphNode_t x = gb.add_kernel(ob, (const void *)k_outer<T, B, W, false>, grid, block, a_body, nullptr, 0);
                 if (p.rowpar) x = gb.add_kernel(ob, (const void *)k_rows_A<T, W>, rgrid, block, a_rows_a, &x, 1);
                 x = gb.add_kernel(ob, (const void *)k_update_sI<T, B, W>, grid, block, a_body, &x, 1);

@@ -6,8 +6,8 @@
 // iteration n (restated from the shifted-Krylov mathematics; rt = S r is the
 // residual of the original equation):
 //   A : u_n = z_s rt_n - H r_n + beta_{n-1} u_{n-1} = (z_s S - H) p_n, the image
-//       of p_n = r_n + beta_{n-1} p_{n-1}; mu_n = p_n^T u_n (S = I: r_n^T u_n;
-//       FP32 panels: S p_n by recurrence and u = z_s S p_n - H p_n);
+//       of p_n = r_n + beta_{n-1} p_{n-1}; mu_n = p_n^T u_n
+//       (FP32 panels: S p_n by recurrence and u = z_s S p_n - H p_n);
 //                                                     (one BSR product with H)
 //       per (slot, shift): pi rotation, residual test, p^m_n on the kept rows;
 //       last CTA: alpha_n = rho_n / mu_n, column done/breakdown, panel done.
@@ -120,7 +120,7 @@ struct Panel {
     int32_t s_unit;   // every diagonal block of S is the identity
     int64_t n_brows;
     // panel vectors [n_rows][W] complex T
-    T *R[2], *RT, *P[2], *SP, *U, *Tv, *Av; // P[1], SP: FP32 panels; P[0]: FP32 or S != I (null otherwise)
+    T *R[2], *RT, *P[2], *SP, *U, *Tv, *Av; // P[1], SP: FP32 panels only (null otherwise)
     typename DirOf<T>::type *D[2]; // inner CG directions (FP32 for df panels)
     // inner solve by refinement (df panels with S): FP32 sweep residual, sweep
     // correction and product S d, and an FP32 copy of S's values

@@ -166,7 +166,7 @@ __global__ void k_validate_bsr(const int64_t *rp, const int32_t *ci, int64_t n_b
 
 // A checking kernel's result reaches the host without an allocation, a memset or
 // a copy: check_words() gives (once per context) three device words and a pinned
-// host word; the kernel ORs what it finds into words[0] and its last CTA calls
+// host word (of 512 pinned bytes, whose rest serves other small results); the kernel ORs what it finds into words[0] and its last CTA calls
 // publish_check, which writes the result to words[2] (for kernels queued behind
 // it) and to the host word, and clears the others for the next check.
 // check_wait() records an event behind the kernel, waits for it and returns the

@@ -115,7 +115,7 @@ int check_words(tb_ctx *ctx, int **words, int **host) {
         int *d = nullptr;
         TB_CUDA_TRY(ctx, cudaMalloc((void **)&d, 4 * sizeof(int)));
         cudaError_t e = cudaMemset(d, 0, 4 * sizeof(int));
-        if (e == cudaSuccess) e = cudaHostAlloc((void **)&ctx->chk_host, sizeof(int), cudaHostAllocPortable);
+        if (e == cudaSuccess) e = cudaHostAlloc((void **)&ctx->chk_host, 512, cudaHostAllocPortable);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->chk_ev, cudaEventDisableTiming);
         // the memset ran on the legacy stream, which a caller's non-blocking stream does not wait for
         if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
