@@ -280,15 +280,15 @@ __device__ __forceinline__ Layout make_layout(int lanes, int cpt, int64_t units)
 __device__ __forceinline__ int pow2_le32(int n) { return n >= 32 ? 32 : (1 << (31 - __clz(n))); }
 
 // K sums per slot: threads -> CTA (part[(slot * K + k) * grid + CTA]).
-template <typename T, int K>
-__device__ __forceinline__ void engine_partials(Acc<T> (&acc)[K], const Layout &l, void *part,
+template <typename T, int K, int CPT = 1>
+__device__ __forceinline__ void engine_partials(Acc<T> (&acc)[CPT * K], const Layout &l, void *part,
                                                 typename Acc<T>::P *sp) {
     typedef typename Acc<T>::P P;
     if (l.team < l.teams) // (an idle slot's sums are zero)
 #pragma unroll
-        for (int k = 0; k < K; ++k) sp[(l.team * l.lanes + l.lane) * K + k] = acc[k].pack();
+        for (int k = 0; k < CPT * K; ++k) sp[(l.team * l.lanes + l.lane) * CPT * K + k] = acc[k].pack();
     __syncthreads();
-    const int rows = l.lanes * K, R = rows >= NT ? 1 : pow2_le32(NT / rows), per = NT / R;
+    const int rows = l.lanes * CPT * K, R = rows >= NT ? 1 : pow2_le32(NT / rows), per = NT / R;
     const int sub = threadIdx.x % R;
     for (int q0 = 0; q0 < rows; q0 += per) {
         const int q = q0 + threadIdx.x / R;
@@ -342,7 +342,7 @@ struct EngineRun {
     const Panel<T> &p;
     unsigned gen;
     struct Smem {
-        typename Acc<T>::P sp[NT * 3];
+        typename Acc<T>::P sp[NT * 3 * (RPT > 1 && HAS_S ? 2 : 1)];
         ColState col[MAX_W]; // the last arriver's copy
         double red[MAX_W * 3], rho[MAX_W * 2];
         unsigned flags;
@@ -657,7 +657,54 @@ struct EngineRun {
     // ------------------------------------------------------------ refinement pass
     // mode 0: y = sigma c, t = rt - S y (first pass); 1: y += sigma c, t -= S sigma c;
     // 2: as 1 with S c and the residual in FP32 (the correction is small, see ENGINE_LIGHT).
+    // The pass in FP32 for kernels with the rows of a block in a thread: two slots a
+    // thread halve the loads of S and of the index arrays.
+    __device__ void phase_R32x2() {
+        const Layout g = make_layout(W / 2, 2, units);
+        const float *c32 = e.X[e.terms & 1];
+        Acc<T> acc[6];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) acc[k].zero();
+        if (g.c >= 0) {
+            const SlotScalars<T> *sc = e.sc + g.c;
+            const T sig[2] = {sc[0].sig, sc[1].sig};
+            const float ratio[2] = {sc[0].ratio, sc[1].ratio};
+            for (int64_t u = g.u0; u < units; u += g.step) {
+                int64_t br;
+                int i0;
+                unit_rows(u, br, i0);
+                cpx<float> sf[RPT][2];
+                rows_product<float, B, RPT, float, 2>(p.s_rp, p.s_ci, p.s_val32, br, i0, c32, W, g.c, p.s_unit, sf, Range{-1, 0});
+#pragma unroll
+                for (int i = 0; i < RPT; ++i) {
+                    const int64_t o = (br * B + i0 + i) * W + g.c;
+                    const float4 c4 = *reinterpret_cast<const float4 *>(c32 + 2 * o), b4 = *reinterpret_cast<const float4 *>(p.T32 + 2 * o);
+                    const float c[4] = {c4.x, c4.y, c4.z, c4.w}, b[4] = {b4.x, b4.y, b4.z, b4.w};
+                    float t[4];
+#pragma unroll
+                    for (int q = 0; q < 2; ++q) {
+                        const cpx<T> rt = ld1(p.RT, o + q);
+                        cpx<T> y = ld1(p.R[0], o + q);
+                        y = mk(scaled_add(sig[q], c[2 * q], y.re), scaled_add(sig[q], c[2 * q + 1], y.im));
+                        st1(p.R[0], o + q, y);
+                        const float tr = b[2 * q] - sf[i][q].re, ti = b[2 * q + 1] - sf[i][q].im;
+                        t[2 * q] = tr * ratio[q], t[2 * q + 1] = ti * ratio[q];
+                        acc[3 * q].add(tr * tr + ti * ti);
+                        acc[3 * q + 1].add(y.re * rt.re);
+                        acc[3 * q + 1].add(-(y.im * rt.im));
+                        acc[3 * q + 2].add(y.re * rt.im);
+                        acc[3 * q + 2].add(y.im * rt.re);
+                    }
+                    *reinterpret_cast<float4 *>(p.T32 + 2 * o) = make_float4(t[0], t[1], t[2], t[3]);
+                }
+            }
+        }
+        engine_partials<T, 3, 2>(acc, g, p.part, s.sp);
+    }
     __device__ void phase_R(int mode) {
+        if constexpr (RPT > 1 && HAS_S) {
+            if (mode == 2 && W % 2 == 0) return phase_R32x2();
+        }
         const float *c32 = e.X[e.terms & 1];
         Acc<T> acc[3];
         acc[0].zero(), acc[1].zero(), acc[2].zero();
