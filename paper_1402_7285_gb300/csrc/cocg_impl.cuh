@@ -22,7 +22,6 @@ __device__ ColState fresh_column(const Panel<T> &p, int64_t col) {
     ColState C;
     memset(&C, 0, sizeof(C));
     C.alpha = mk(0.0, 0.0);
-    C.alpha_prev = mk(1.0, 0.0);
     C.beta_prev = mk(0.0, 0.0);
     C.rho = mk(1.0, 0.0); // S = I: rho_0 = e_j^T e_j; S != I: replaced by the init pass
     C.rn2 = 1.0;
@@ -49,7 +48,7 @@ __device__ ColState fresh_column(const Panel<T> &p, int64_t col) {
 
 __device__ __forceinline__ ShiftState fresh_shift() {
     ShiftState S;
-    S.pi = S.pi_prev = S.pi_next = mk(1.0, 0.0);
+    S.pi = S.pi_prev = S.pi_next = S.ipi = mk(1.0, 0.0);
     S.alpha_s = mk(0.0, 0.0);
     S.resid = 1.0;
     S.active = 1;
@@ -180,19 +179,24 @@ __device__ __forceinline__ PairA pair_coef_A(const Panel<T> &p, int q, int n) {
     r.eta = 0.0;
     ColState &C = p.col[q / p.nz];
     ShiftState &S = p.sh[q];
-    if (C.done || !S.active) return r;
-    S.pi_prev = S.pi;
-    S.pi = S.pi_next;
+    // loaded before the first branch (L2 trips), and no division: B left 1 / pi_n
+    const c64 pi_prev = S.pi, pi = S.pi_next, ipi = S.ipi, beta = C.beta_prev;
+    const double rn2 = C.rn2;
+    const int done = C.done, active = S.active;
+    if (done || !active) return r;
+    S.pi_prev = pi_prev;
+    S.pi = pi;
     double res;
     if (p.qmr) {
-        const double w2inv = cabs2(S.pi) / sqrt(cabs2(C.rho)); // 1 / omega_n^2
+        const double w2inv = cabs2(pi) / sqrt(cabs2(C.rho)); // 1 / omega_n^2
         if (S.qinv == 0.0) S.qinv0 = w2inv;
-        S.qinv += w2inv;
-        r.eta = w2inv / S.qinv;
-        res = sqrt(S.qinv0 / S.qinv);
+        const double qinv = S.qinv + w2inv, iq = 1.0 / qinv;
+        S.qinv = qinv;
+        r.eta = w2inv * iq;
+        res = sqrt(S.qinv0 * iq);
         r.on = 2; // smoothing update of the kept rows
     } else {
-        res = sqrt(C.rn2) / sqrt(cabs2(S.pi));
+        res = sqrt(rn2) * sqrt(cabs2(ipi));
     }
     S.resid = res;
     if (res <= p.tol) {
@@ -200,9 +204,9 @@ __device__ __forceinline__ PairA pair_coef_A(const Panel<T> &p, int q, int n) {
         S.conv_it = n;
         atomicSub(&C.n_active, 1);
     } else {
-        const c64 ratio = cdiv(S.pi_prev, S.pi);
-        r.b = (ratio * ratio) * C.beta_prev;
-        r.a = cdiv(mk(1.0, 0.0), S.pi);
+        const c64 ratio = pi_prev * ipi;
+        r.b = (ratio * ratio) * beta;
+        r.a = ipi;
         r.on |= 1;
     }
     return r;
@@ -264,11 +268,12 @@ __device__ __forceinline__ bool pair_coef_B(const Panel<T> &p, int q, c64 &as) {
     as = mk(0.0, 0.0);
     ColState &C = p.col[q / p.nz];
     ShiftState &S = p.sh[q];
-    if (C.done || !S.active) return false;
-    const c64 sig = p.z[q % p.nz] - C.zs;
-    const c64 coef = cdiv(C.alpha * C.beta_prev, C.alpha_prev);
-    const c64 pn = (mk(1.0, 0.0) + C.alpha * sig) * S.pi + coef * (S.pi - S.pi_prev);
-    as = cdiv(S.pi, pn) * C.alpha;
+    const c64 sig = p.z[q % p.nz] - C.zs, al = C.alpha, boa = C.boa, pi = S.pi, pi_prev = S.pi_prev;
+    const int done = C.done, active = S.active;
+    if (done || !active) return false;
+    const c64 pn = (mk(1.0, 0.0) + al * sig) * pi + (al * boa) * (pi - pi_prev);
+    const c64 ipn = cinv(pn);
+    as = (pi * ipn) * al;
     if (!cfinite(pn) || (pn.re == 0.0 && pn.im == 0.0) || !cfinite(as)) {
         S.active = 0;
         S.resid = nan("");
@@ -277,6 +282,7 @@ __device__ __forceinline__ bool pair_coef_B(const Panel<T> &p, int q, c64 &as) {
         return false;
     }
     S.pi_next = pn;
+    S.ipi = ipn;
     S.alpha_s = as;
     return true;
 }
@@ -414,7 +420,7 @@ __device__ bool finish_alpha(const Panel<T> &p, int W, const double *red, ColSta
             st = TB_COL_MAX_ITER;
         c64 a = mk(0.0, 0.0);
         if (st < 0) {
-            a = cdiv(rho, mu);
+            a = rho * cinv(mu);
             if (!cfinite(a)) st = TB_COL_NONFINITE;
         }
         if (st >= 0) {
@@ -523,7 +529,7 @@ __device__ bool finish_alpha(const Panel<T> &p, int W, const double *red, ColSta
             for (int m = 0; m < p.nz; ++m) {
                 ShiftState &S = p.sh[(int64_t)c * p.nz + m];
                 if (!S.active) continue;
-                S.pi = S.pi_prev = S.pi_next = mk(1.0, 0.0);
+                S.pi = S.pi_prev = S.pi_next = S.ipi = mk(1.0, 0.0);
                 S.resid = 1.0;
                 for (int k = 0; k < C.n_ent; ++k) {
                     p.xs[((int64_t)c * KM + k) * p.nz + m] = mk(0.0, 0.0);
@@ -637,16 +643,16 @@ __device__ void finish_outer(const Panel<T> &p, int W, const double *rho_next, i
             continue;
         }
         if (restart) { // first iteration of the new seed follows
-            C.beta_prev = mk(0.0, 0.0);
-            C.alpha_prev = mk(1.0, 0.0);
+            C.beta_prev = C.boa = mk(0.0, 0.0);
             C.rho = rn;
             C.restart = 0;
             C.fresh = 0;
             C.iters = its + 1;
             continue;
         }
-        C.beta_prev = cdiv(rn, rho);
-        C.alpha_prev = alpha;
+        const c64 be = rn * cinv(rho);
+        C.beta_prev = be;
+        C.boa = be * cinv(alpha);
         C.rho = rn;
         C.iters = its + 1;
     }

@@ -32,8 +32,8 @@ namespace tbgf {
 struct ColState {
     c64 rho;        // rho_n  = r_n^T rt_n
     c64 alpha;      // alpha_n (0 when the column is done)
-    c64 alpha_prev; // alpha_{n-1}
     c64 beta_prev;  // beta_{n-1}
+    c64 boa;        // beta_{n-1} / alpha_{n-1}
     c64 rho_next;   // rho_{n+1} (between B/C row work and finalize)
     double rn2;     // ||rt_n||^2
     double in_rr;   // inner CG: t^H t
@@ -66,6 +66,7 @@ __host__ __device__ __forceinline__ double safe_scale(double norm2) {
 
 struct ShiftState {
     c64 pi, pi_prev, pi_next; // pi_{n-1}, pi_{n-2}, pi_n at the start of A(n)
+    c64 ipi;                  // 1 / pi_next (B has the inverse; A needs it)
     c64 alpha_s;
     double resid;
     int32_t active, conv_it;

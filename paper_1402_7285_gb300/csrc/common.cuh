@@ -49,6 +49,17 @@ __host__ __device__ __forceinline__ cpx<T> cdiv(cpx<T> a, cpx<T> b) {
         return mk((a.re * r + a.im) / d, (a.im * r - a.re) / d);
     }
 }
+// 1 / z with one division (an FP64 division takes 436 cycles on GB300, and Smith's two
+// branches run one after the other in a warp whose lanes differ): z is scaled by a
+// power of two to a largest component in [1, 2), so |z|^2 neither over- nor
+// underflows.  Zero and non-finite z give non-finite results.
+__device__ __forceinline__ cpx<double> cinv(cpx<double> z) {
+    const int e = __double2hiint(fmax(fabs(z.re), fabs(z.im))) & 0x7ff00000;
+    const double s = __hiloint2double(0x7fe00000 - e, 0);
+    const double x = z.re * s, y = z.im * s;
+    const double q = s / fma(x, x, y * y);
+    return mk(x * q, -y * q);
+}
 template <typename T>
 __host__ __device__ __forceinline__ T cabs2(cpx<T> a) { return a.re * a.re + a.im * a.im; }
 __host__ __device__ __forceinline__ bool cfinite(c64 a) { return isfinite(a.re) && isfinite(a.im); }
