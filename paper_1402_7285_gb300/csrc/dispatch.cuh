@@ -46,5 +46,7 @@ bool dispatch_tbw(F &f, bool f32, int b, int W) {
 
 // FP64 matrix values -> the precision's value type (FP32 or df) in dst
 void convert_values(int precision, const double *src, void *dst, int64_t n, cudaStream_t s);
+// the same with each b x b block transposed (FP32 and df)
+void convert_values_t(int precision, const double *src, void *dst, int64_t n, int b, cudaStream_t s);
 
 } // namespace tbgf

@@ -1,5 +1,5 @@
 // shifted_cocg_solve_local: host driver (kernels in local_impl.cuh).
-#include "local_impl.cuh"
+#include "local_engine.cuh"
 
 namespace tbgf {
 
@@ -8,12 +8,13 @@ __global__ void k_copy_z_local(const double *z, c64 *zc, int nz) {
 }
 
 __global__ void k_same_pattern(const int64_t *a_rp, const int32_t *a_ci, const int64_t *b_rp, const int32_t *b_ci,
-                               int64_t n, int64_t nnzb, int *bad) {
+                               int64_t n, int64_t nnzb, int *words, int *host) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i <= n; i += stride)
-        if (a_rp[i] != b_rp[i]) atomicOr(bad, 1);
+        if (a_rp[i] != b_rp[i]) atomicOr(words, 1);
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nnzb; i += stride)
-        if (a_ci[i] != b_ci[i]) atomicOr(bad, 1);
+        if (a_ci[i] != b_ci[i]) atomicOr(words, 1);
+    publish_check(words, host);
 }
 
 } // namespace tbgf
@@ -137,10 +138,184 @@ extern "C" int shifted_cocg_solve_local(tb_ctx *ctx, const tb_bsr *H, const tb_b
     if (rc) return rc;
     rc = validate_bsr(ctx, (const int64_t *)d_hrp, (const int32_t *)d_hci, d_hval, H->n_brows, H->nnzb, stream, "H");
     if (rc) return rc;
-    // ---- workspace: per-CTA kept-row states, z, FP32 matrix copies, queue, pattern check
     int sms = 152, dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (has_s) {
+        int *words = nullptr, *host = nullptr, h = 0;
+        rc = check_words(ctx, &words, &host);
+        if (rc) return rc;
+        k_same_pattern<<<152 * 4, 256, 0, stream>>>((const int64_t *)d_hrp, (const int32_t *)d_hci,
+                                                    (const int64_t *)d_srp, (const int32_t *)d_sci, H->n_brows,
+                                                    H->nnzb, words, host);
+        rc = check_wait(ctx, stream, &h);
+        if (rc) return rc;
+        TB_CHECK(ctx, h == 0, TB_ERR_ARG, "S must have H's block pattern");
+    }
+    // seed shift: median real part
+    std::vector<int> idx(n_z);
+    for (int i = 0; i < n_z; ++i) idx[i] = i;
+    std::stable_sort(idx.begin(), idx.end(), [&](int x, int y) { return h_z[2 * x] < h_z[2 * y]; });
+    const int seed = opts.seed_shift >= 0 ? opts.seed_shift : idx[n_z / 2];
+    LocalArgs<double> la;
+    std::memset(&la, 0, sizeof(la));
+    la.h_rp = (const int64_t *)d_hrp;
+    la.h_ci = (const int32_t *)d_hci;
+    la.n_brows = H->n_brows;
+    la.nz = n_z;
+    la.zs = mk(h_z[2 * seed], h_z[2 * seed + 1]);
+    la.rhs = (const int64_t *)d_rhs;
+    la.sub_ptr = (const int64_t *)d_sptr;
+    la.sub_atoms = (const int32_t *)d_atoms;
+    la.optr = (const int64_t *)d_optr;
+    la.orows = (const int64_t *)d_orows;
+    la.dmax = dmax;
+    la.tol = opts.tol;
+    la.inner_tol = opts.inner_tol > 0.0 ? opts.inner_tol : std::max(1e-3 * opts.tol, mixed ? 1e-7 : (lowp ? 1e-12 : 1e-13));
+    la.max_iter = opts.max_iter;
+    la.inner_max = opts.inner_max > 0 ? opts.inner_max : 40;
+    // seed residual below which df64 no longer carries the harder shifts
+    // (restart with a new seed); FP64 converges without, FP32 never gets there
+    la.stall2 = opts.precision == TB_PREC_DF64 ? 1e-20 : 0.0;
+    la.G = (c64 *)d_G;
+    la.iters = (int32_t *)d_iters;
+    la.resid = (double *)d_resid;
+    la.status = (int32_t *)d_status;
+
+    auto finish_call = [&](const unsigned long long *dev_stat) -> int {
+        if (opts.stats) {
+            unsigned long long st2[2];
+            TB_CUDA_TRY(ctx, cudaMemcpy(st2, dev_stat, sizeof(st2), cudaMemcpyDeviceToHost));
+            opts.stats[0] = (int64_t)st2[0];
+            opts.stats[1] = (int64_t)st2[1];
+        }
+        std::vector<int32_t> stv(n_rhs);
+        TB_CUDA_TRY(ctx, cudaMemcpy(stv.data(), d_status, sizeof(int32_t) * n_rhs, cudaMemcpyDeviceToHost));
+        int r = stg.finish();
+        if (r) return r;
+        int warn = 0;
+        for (int32_t s : stv) {
+            if (s == TB_COL_MAX_ITER) warn |= TB_WARN_MAX_ITER;
+            if (s == TB_COL_BREAKDOWN) warn |= TB_WARN_BREAKDOWN;
+            if (s == TB_COL_NONFINITE) warn |= TB_WARN_NONFINITE;
+        }
+        return warn;
+    };
+
+    // ---- FP64 and df vectors, with S when its spectrum allows Chebyshev sweeps: local_engine.cuh.  FP32 vectors
+    // and other S: k_local, below.
+    LocalArgs2<double> la2;
+    std::memset(&la2, 0, sizeof(la2));
+    bool sweeps = !mixed;
+    // (the sweeps make the tighter target of the df panel solver cheap here too)
+    const double cg_tol = la.inner_tol;
+    if (opts.inner_tol <= 0.0 && lowp && !mixed) la.inner_tol = std::max(1e-5 * opts.tol, 1e-12);
+    if (sweeps && has_s) {
+        double lo = 1, hi = 0;
+        rc = spectral_bounds(ctx, (const int64_t *)d_srp, (const int32_t *)d_sci, (const double *)d_sval, H->n_brows, b,
+                             sms, stream, &lo, &hi);
+        if (rc) return rc;
+        sweeps = chebyshev_terms(lo, hi, la.inner_tol, la.inner_max, false, la2);
+    }
+    if (sweeps) {
+        int optin2 = 0;
+        cudaDeviceGetAttribute(&optin2, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        LocalLaunch2 L{};
+        L.ctx = ctx, L.has_s = has_s, L.sms = sms, L.probe = true;
+        if (!(lowp ? launch_local2_df(L, b) : launch_local2_f64(L, b)))
+            return set_error(ctx, TB_ERR_UNSUPPORTED, "no local solver variant");
+        if (L.rc) return L.rc;
+        L.probe = false;
+        L.static_bytes = L.static_smem;
+        const size_t limit = (size_t)optin2 - L.static_smem;
+        L.static_smem = (int)limit; // the most dynamic shared memory of a launch
+        size_t off = 0;
+        auto take = [&](size_t bytes) {
+            size_t o = off;
+            off = align_up(off + bytes, 256);
+            return o;
+        };
+        // Threads of a CTA: about two rows each of the largest subspace, 1024 threads to an SM.  The own-row
+        // vectors leave shared memory when more CTAs fit an SM without them (largest 686 rows with overlap: 92 us
+        // an iteration in one CTA per SM); a subspace that still leaves room for one CTA only gets 1024 threads.
+        const int64_t maxr = (int64_t)maxa * b;
+        L.threads = maxr > 448 ? 512 : (maxr > 160 ? 256 : 128);
+        const size_t fixed = local_smem(maxa, dmax, max_kept, n_z, has_s, b, 16, false);
+        TB_CHECK(ctx, fixed <= limit, TB_ERR_SIZE, "local subspace needs %zu bytes of shared memory (limit %zu)", fixed, limit);
+        const size_t ga = local2_gather(has_s, 16, maxr), ow = local2_own(has_s, 16, maxr);
+        int best = 0;
+        for (int mode = 0; mode < 3; ++mode) {
+            const size_t sm = fixed + (mode < 2 ? ga : 0) + (mode < 1 ? ow : 0);
+            const int fit = sm > limit ? 0 : (int)std::min<size_t>(1024 / L.threads, (size_t)optin2 / (sm + L.static_bytes + 1024));
+            if (mode == 2 ? best > 0 : fit <= best) continue;
+            best = std::max(fit, 1);
+            la2.own_global = mode;
+            L.smem = sm;
+        }
+        if (best == 1 && maxr > 1024) L.threads = 1024;
+        L.grid = (int)std::min<int64_t>(n_rhs, (int64_t)sms * (1024 / L.threads));
+        const size_t o_scr = take(sizeof(c64) * 2 * (size_t)max_kept * n_z * L.grid);
+        const size_t o_gvec = la2.own_global ? take((ow + (la2.own_global == 2 ? ga : 0)) * L.grid) : 0;
+        const size_t o_zc = take(sizeof(c64) * n_z), o_q = take(sizeof(unsigned long long) * 8);
+        const size_t o_h = lowp ? take(sizeof(double) * H->nnzb * bb) : 0;
+        const size_t o_s = lowp && has_s ? take(sizeof(double) * S->nnzb * bb) : 0;
+        const size_t o_sf = has_s ? take(sizeof(float) * S->nnzb * bb) : 0;
+        void *wsp = nullptr;
+        rc = ws_get(ctx, WS_SOLVE_SMALL, off, &wsp);
+        if (rc) return rc;
+        char *ws = (char *)wsp;
+        TB_CUDA_TRY(ctx, cudaMemsetAsync(ws + o_q, 0, sizeof(unsigned long long) * 8, stream));
+        k_copy_z_local<<<1, 256, 0, stream>>>((const double *)d_z, (c64 *)(ws + o_zc), n_z);
+        const int64_t nv = H->nnzb * bb;
+        auto convert = [&](int prec, const void *src, size_t o) {
+            if (b == 9 && lowp)
+                convert_values_t(prec, (const double *)src, ws + o, nv, b, stream);
+            else
+                convert_values(prec, (const double *)src, ws + o, nv, stream);
+        };
+        la.h_val = (const double *)d_hval;
+        la.s_val = has_s ? (const double *)d_sval : nullptr;
+        if (lowp) {
+            convert(TB_PREC_DF64, d_hval, o_h);
+            la.h_val = (const double *)(ws + o_h);
+            if (has_s) {
+                convert(TB_PREC_DF64, d_sval, o_s);
+                la.s_val = (const double *)(ws + o_s);
+            }
+        }
+        if (has_s) {
+            if (b == 9) // FP32 blocks of 9 x 9 are transposed for FP64 vectors too
+                convert_values_t(TB_PREC_MIXED, (const double *)d_sval, ws + o_sf, nv, b, stream);
+            else
+                convert_values(TB_PREC_MIXED, (const double *)d_sval, ws + o_sf, nv, stream);
+        }
+        TB_CUDA_TRY(ctx, cudaGetLastError());
+        unsigned long long *words = (unsigned long long *)(ws + o_q); // queue, statistics, fault
+        la.z = (const c64 *)(ws + o_zc);
+        la.order = (const int64_t *)d_order;
+        la.n = n_rhs;
+        la.maxa = maxa;
+        la.max_kept = max_kept;
+        la.scratch = (c64 *)(ws + o_scr);
+        la.gvec = la2.own_global ? (void *)(ws + o_gvec) : nullptr;
+        la.queue = words;
+        la.stat = words + 1;
+        la2.a = la;
+        la2.s_val32 = (const float *)(ws + o_sf);
+        la2.fail = (int32_t *)(words + 3);
+        L.args = la2;
+        L.cols = n_rhs;
+        L.stream = stream;
+        lowp ? launch_local2_df(L, b) : launch_local2_f64(L, b);
+        if (L.rc) return L.rc;
+        int32_t fail = 0;
+        TB_CUDA_TRY(ctx, cudaMemcpyAsync(&fail, la2.fail, sizeof(fail), cudaMemcpyDeviceToHost, stream));
+        TB_CUDA_TRY(ctx, cudaStreamSynchronize(stream));
+        if (!fail) return finish_call(la.stat);
+    }
+
+    la.inner_tol = cg_tol;
+    // ---- workspace: per-CTA kept-row states, z, FP32 matrix copies, queue
     const int grid = sms * 2;
     size_t off = 0;
     auto take = [&](size_t bytes) {
@@ -165,16 +340,6 @@ extern "C" int shifted_cocg_solve_local(tb_ctx *ctx, const tb_bsr *H, const tb_b
     if (rc) return rc;
     char *ws = (char *)wsp;
     TB_CUDA_TRY(ctx, cudaMemsetAsync(ws + o_q, 0, sizeof(unsigned long long) * 4, stream));
-    if (has_s) {
-        int *flag = (int *)(ws + o_q) + 6;
-        k_same_pattern<<<152 * 4, 256, 0, stream>>>((const int64_t *)d_hrp, (const int32_t *)d_hci,
-                                                     (const int64_t *)d_srp, (const int32_t *)d_sci, H->n_brows,
-                                                     H->nnzb, flag);
-        int h = 0;
-        TB_CUDA_TRY(ctx, cudaMemcpyAsync(&h, flag, sizeof(int), cudaMemcpyDeviceToHost, stream));
-        TB_CUDA_TRY(ctx, cudaStreamSynchronize(stream));
-        TB_CHECK(ctx, h == 0, TB_ERR_ARG, "S must have H's block pattern");
-    }
     k_copy_z_local<<<1, 256, 0, stream>>>((const double *)d_z, (c64 *)(ws + o_zc), n_z);
     const void *hval = d_hval, *sval = d_sval;
     if (lowp) {
@@ -185,46 +350,17 @@ extern "C" int shifted_cocg_solve_local(tb_ctx *ctx, const tb_bsr *H, const tb_b
             sval = ws + o_s32;
         }
     }
-    // seed shift: median real part
-    std::vector<int> idx(n_z);
-    for (int i = 0; i < n_z; ++i) idx[i] = i;
-    std::stable_sort(idx.begin(), idx.end(), [&](int x, int y) { return h_z[2 * x] < h_z[2 * y]; });
-    const int seed = opts.seed_shift >= 0 ? opts.seed_shift : idx[n_z / 2];
-    LocalArgs<double> la;
-    std::memset(&la, 0, sizeof(la));
-    la.h_rp = (const int64_t *)d_hrp;
-    la.h_ci = (const int32_t *)d_hci;
     la.h_val = (const double *)hval;
     la.s_val = has_s ? (const double *)sval : nullptr;
-    la.n_brows = H->n_brows;
     la.z = (const c64 *)(ws + o_zc);
-    la.nz = n_z;
-    la.zs = mk(h_z[2 * seed], h_z[2 * seed + 1]);
-    la.rhs = (const int64_t *)d_rhs;
-    la.sub_ptr = (const int64_t *)d_sptr;
-    la.sub_atoms = (const int32_t *)d_atoms;
-    la.optr = (const int64_t *)d_optr;
-    la.orows = (const int64_t *)d_orows;
     la.order = (const int64_t *)d_order;
     la.n = n_rhs;
     la.maxa = maxa;
-    la.dmax = dmax;
     la.max_kept = max_kept;
     la.scratch = (c64 *)(ws + o_scr);
     la.gvec = vec_global ? (void *)(ws + o_gvec) : nullptr;
     la.queue = (unsigned long long *)(ws + o_q);
     la.stat = (unsigned long long *)(ws + o_q) + 1;
-    la.tol = opts.tol;
-    la.inner_tol = opts.inner_tol > 0.0 ? opts.inner_tol : std::max(1e-3 * opts.tol, mixed ? 1e-7 : (lowp ? 1e-12 : 1e-13));
-    la.max_iter = opts.max_iter;
-    la.inner_max = opts.inner_max > 0 ? opts.inner_max : 40;
-    // seed residual below which df64 no longer carries the harder shifts
-    // (restart with a new seed); FP64 converges without, FP32 never gets there
-    la.stall2 = opts.precision == TB_PREC_DF64 ? 1e-20 : 0.0;
-    la.G = (c64 *)d_G;
-    la.iters = (int32_t *)d_iters;
-    la.resid = (double *)d_resid;
-    la.status = (int32_t *)d_status;
     LocalLaunch L{ctx, la, has_s, grid, stream};
     const bool launched = opts.precision == TB_PREC_FP64    ? launch_local_f64(L, b)
                           : opts.precision == TB_PREC_MIXED ? launch_local_f32(L, b)
@@ -232,21 +368,5 @@ extern "C" int shifted_cocg_solve_local(tb_ctx *ctx, const tb_bsr *H, const tb_b
     if (!launched) return set_error(ctx, TB_ERR_UNSUPPORTED, "no local solver variant");
     if (L.rc) return L.rc;
     TB_CUDA_TRY(ctx, cudaStreamSynchronize(stream));
-    if (opts.stats) {
-        unsigned long long st2[2];
-        TB_CUDA_TRY(ctx, cudaMemcpy(st2, la.stat, sizeof(st2), cudaMemcpyDeviceToHost));
-        opts.stats[0] = (int64_t)st2[0];
-        opts.stats[1] = (int64_t)st2[1];
-    }
-    std::vector<int32_t> stv(n_rhs);
-    TB_CUDA_TRY(ctx, cudaMemcpy(stv.data(), d_status, sizeof(int32_t) * n_rhs, cudaMemcpyDeviceToHost));
-    rc = stg.finish();
-    if (rc) return rc;
-    int warn = 0;
-    for (int32_t s : stv) {
-        if (s == TB_COL_MAX_ITER) warn |= TB_WARN_MAX_ITER;
-        if (s == TB_COL_BREAKDOWN) warn |= TB_WARN_BREAKDOWN;
-        if (s == TB_COL_NONFINITE) warn |= TB_WARN_NONFINITE;
-    }
-    return warn;
+    return finish_call(la.stat);
 }

@@ -101,6 +101,17 @@ __global__ void __launch_bounds__(SNT) k_convert(const double *src, T *dst, int6
     convert_span(src, dst, n);
 }
 
+// dst block (j, i) = src block (i, j), b x b blocks: the rows of a block become neighbours
+template <typename T>
+__global__ void __launch_bounds__(SNT) k_convert_t(const double *__restrict__ src, T *__restrict__ dst, int64_t n, int b) {
+    const int bb = b * b;
+    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t k = t / bb;
+        const int r = (int)(t - k * bb), j = r / b, i = r - j * b;
+        cvt_to(src[k * bb + i * b + j], dst[t]);
+    }
+}
+
 // First launch of a product: the structure check of A and, for FP32 and df, the
 // conversion of A's values and of X.
 template <typename T>
@@ -323,6 +334,13 @@ void convert_values(int precision, const double *src, void *dst, int64_t n, cuda
         k_convert<float><<<g, SNT, 0, s>>>(src, (float *)dst, n);
     else if (precision == TB_PREC_DF64)
         k_convert<df><<<g, SNT, 0, s>>>(src, (df *)dst, n);
+}
+void convert_values_t(int precision, const double *src, void *dst, int64_t n, int b, cudaStream_t s) {
+    const int g = (int)std::max<int64_t>(1, std::min<int64_t>((n + SNT - 1) / SNT, 152 * 8));
+    if (precision == TB_PREC_MIXED)
+        k_convert_t<float><<<g, SNT, 0, s>>>(src, (float *)dst, n, b);
+    else
+        k_convert_t<df><<<g, SNT, 0, s>>>(src, (df *)dst, n, b);
 }
 } // namespace tbgf
 

@@ -31,15 +31,15 @@ def _bsr(b):
     return tb.Bsr(b.n_brows, b.bdim, b.row_ptr, b.col_idx, b.val).to(DEV)
 
 
-def _check(H, S, n_cols, prec, solver=COCG, full=False, panel_w=0, seed_shift=-1, tol=1e-11):
-    M = H.n_rows
+def _check(H, S, n_cols, prec, solver=COCG, full=False, panel_w=0, seed_shift=-1, tol=1e-11, inner_max=0):
+    M = H.n_brows * H.bdim
     cols = np.unique(np.linspace(0, M - 1, n_cols).astype(np.int64))
     rl = [np.arange(M) if full else systems.block_pattern_rows(H, j) for j in cols]
     ptr, rows = out_layout(rl)
     z = wl.midpoint_shifts(7, -8.0, 6.0, 0.2)
     with tb.Context() as ctx:
         r = tb.solve(ctx, _bsr(H), None if S is None else _bsr(S), z, cols, ptr, rows, tol=tol, precision=prec,
-                     solver=solver, panel_w=panel_w, seed_shift=seed_shift)
+                     solver=solver, panel_w=panel_w, seed_shift=seed_shift, inner_max=inner_max)
         assert r.rc == 0 and np.all(r.status.cpu().numpy() == tb.TB_COL_CONVERGED)
         G = r.G.cpu().numpy()
     ex = dense.green_lu(H.to_dense(), None if S is None else S.to_dense(), z, cols)
@@ -80,10 +80,10 @@ def test_wide_overlap_spectrum_takes_conjugate_gradients(prec):
     """S = D S0 D with D from 0.3 to 2 keeps S positive definite but spreads its spectrum."""
     o = systems.build_system(wl.scaled(wl.C2_SYSTEM, L=3), 3)
     S = o.S
-    d = np.random.default_rng(1).uniform(0.3, 2.0, S.n_rows).reshape(S.n_brows, S.bdim)
+    d = np.random.default_rng(1).uniform(0.3, 2.0, (S.n_brows, S.bdim))
     br = np.repeat(np.arange(S.n_brows), np.diff(S.row_ptr))
     S.val[:] = S.val * d[br][:, :, None] * d[S.col_idx][:, None, :]
-    _check(o.H, S, 5, prec)
+    _check(o.H, S, 5, prec, inner_max=200)   # a condition number near 100: more steps than the default 40
 
 
 def test_seed_at_the_edge_of_the_spectrum_leaves_fp32_range():
