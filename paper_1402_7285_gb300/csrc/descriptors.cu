@@ -28,20 +28,41 @@ __device__ __forceinline__ int find_atom(const int32_t *atoms, int n, int64_t g)
     return -1;
 }
 
-// CTA sum of one double (FP64: descriptors are a one-off per column)
-__device__ __forceinline__ double cta_sum_d(double v, double *scratch) {
-    v = warp_sum(v);
-    if ((threadIdx.x & 31) == 0) scratch[threadIdx.x >> 5] = v;
-    __syncthreads();
-    double s = 0.0;
-    if (threadIdx.x == 0) {
-        for (int w = 0; w < DNT / 32; ++w) s += scratch[w];
-        scratch[DNT / 32] = s;
+// CTA sums of K doubles, in v of every thread; two barriers for all K (a sum of its
+// own for each of the 24 numbers cost 29 us a column)
+template <int K>
+__device__ __forceinline__ void cta_sums(double (&v)[K], double (*scratch)[DNT / 32 + 1]) {
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        v[k] = warp_sum(v[k]);
+        if ((threadIdx.x & 31) == 0) scratch[k][threadIdx.x >> 5] = v[k];
     }
     __syncthreads();
-    s = scratch[DNT / 32];
+    if (threadIdx.x < K) {
+        double s = 0.0;
+        for (int w = 0; w < DNT / 32; ++w) s += scratch[threadIdx.x][w];
+        scratch[threadIdx.x][DNT / 32] = s;
+    }
     __syncthreads();
-    return s;
+#pragma unroll
+    for (int k = 0; k < K; ++k) v[k] = scratch[k][DNT / 32];
+}
+
+// sum_j row[j] x[j] added to y in order
+template <int B>
+__device__ __forceinline__ double dot_row(const double *__restrict__ row, const double *x, double y) {
+    if constexpr (B % 2 == 0) { // rows of such blocks are 16-byte aligned
+#pragma unroll
+        for (int q = 0; q < B; q += 2) {
+            const double2 h = __ldg(reinterpret_cast<const double2 *>(row + q));
+            y = fma(h.x, x[q], y);
+            y = fma(h.y, x[q + 1], y);
+        }
+    } else {
+#pragma unroll
+        for (int q = 0; q < B; ++q) y = fma(__ldg(row + q), x[q], y);
+    }
+    return y;
 }
 
 template <int B>
@@ -60,8 +81,8 @@ __global__ void __launch_bounds__(DNT) k_desc(const int64_t *__restrict__ h_rp, 
     int16_t *nbl = reinterpret_cast<int16_t *>(nbk + maxa * dmax);
     int16_t *cnt = nbl + maxa * dmax;
     int16_t *dist = cnt + maxa;
-    __shared__ double scratch[DNT / 32 + 1];
-    __shared__ int s_changed;
+    __shared__ double scratch[5][DNT / 32 + 1];
+    __shared__ int s_shell[6], s_max, s_surf;
     const int tid = threadIdx.x;
     for (int64_t c = blockIdx.x; c < n; c += gridDim.x) {
         const int64_t a0 = sub_ptr[c];
@@ -100,63 +121,43 @@ __global__ void __launch_bounds__(DNT) k_desc(const int64_t *__restrict__ h_rp, 
             __syncthreads();
         }
         const int nrows = nat * B;
-        // --- shell counts, surface fraction
-        double shell[6] = {0, 0, 0, 0, 0, 0};
-        int dmx_local = 0;
+        // --- shell counts, largest hop distance
+        if (tid < 6) s_shell[tid] = 0;
+        if (tid == 6) s_max = 0, s_surf = 0;
+        __syncthreads();
         for (int l = tid; l < nat; l += DNT) {
             const int dd = dist[l];
-            if (dd >= 1 && dd <= 5) shell[dd] += 1.0;
-            dmx_local = max(dmx_local, (int)dd);
+            if (dd >= 1 && dd <= 5) atomicAdd(&s_shell[dd], 1);
+            if (dd > 0) atomicMax(&s_max, dd);
         }
-        double shells[6];
-        for (int s = 1; s <= 5; ++s) shells[s] = cta_sum_d(shell[s], scratch);
-        // max hop distance in the subspace = number of levels actually reached
-        double dm = cta_sum_d(0.0, scratch); // sync point
-        (void)dm;
-        if (tid == 0) s_changed = 0;
-        __syncthreads();
-        atomicMax(&s_changed, dmx_local);
-        __syncthreads();
-        const int dmax_reached = s_changed;
-        double surf = 0.0;
-        for (int l = tid; l < nat; l += DNT) surf += (dist[l] == dmax_reached) ? 1.0 : 0.0;
-        surf = cta_sum_d(surf, scratch);
-        // --- diagonal statistics and row-j sums
-        double dsum = 0, dsq = 0, dmin = 1e300, dmaxv = -1e300, hrow = 0, srow = 0, hjj = 0;
+        // --- diagonal statistics and row-j sums (dsum, dsq, hjj, hrow, srow)
+        double st[5] = {0, 0, 0, 0, 0}, dmin = 1e300, dmaxv = -1e300;
         for (int l = tid; l < nrows; l += DNT) {
             const int lat = l / B, i = l % B;
             for (int s = 0; s < cnt[lat]; ++s) {
-                const int lc = nbl[lat * dmax + s];
-                const int64_t kb = nbk[lat * dmax + s];
-                if (lc == lat) {
-                    const double h = h_val[kb * B * B + i * B + i];
-                    dsum += h;
-                    dsq += h * h;
-                    dmin = fmin(dmin, h);
-                    dmaxv = fmax(dmaxv, h);
-                }
-                if (l == jl) {
-                    for (int q = 0; q < B; ++q) {
-                        const int col = lc * B + q;
-                        if (col == jl) {
-                            hjj = h_val[kb * B * B + i * B + q];
-                            continue;
-                        }
-                        const double h = h_val[kb * B * B + i * B + q];
-                        hrow += h * h;
-                        if (s_val) {
-                            const double sv = s_val[kb * B * B + i * B + q];
-                            srow += sv * sv;
-                        }
-                    }
-                }
+                if (nbl[lat * dmax + s] != lat) continue;
+                const double h = h_val[(int64_t)nbk[lat * dmax + s] * B * B + i * B + i];
+                st[0] += h;
+                st[1] += h * h;
+                dmin = fmin(dmin, h);
+                dmaxv = fmax(dmaxv, h);
             }
         }
-        const double dmean = cta_sum_d(dsum, scratch) / nrows;
-        const double dvar = cta_sum_d(dsq, scratch) / nrows - dmean * dmean;
-        hjj = cta_sum_d(hjj, scratch);
-        hrow = cta_sum_d(hrow, scratch);
-        srow = cta_sum_d(srow, scratch);
+        const int jo = jl % B;
+        for (int e = tid; e < cnt[la] * B; e += DNT) { // row j, an entry a thread
+            const int s = e / B, q = e - s * B, lc = nbl[la * dmax + s];
+            const int64_t at = (int64_t)nbk[la * dmax + s] * B * B + jo * B + q;
+            const double h = h_val[at];
+            if (lc == la && q == jo) {
+                st[2] += h;
+                continue;
+            }
+            st[3] += h * h;
+            if (s_val) {
+                const double sv = s_val[at];
+                st[4] += sv * sv;
+            }
+        }
         // min / max through warp reductions of the negated / plain values
         double mn = dmin, mx = dmaxv;
         for (int o = 16; o > 0; o >>= 1) {
@@ -165,47 +166,52 @@ __global__ void __launch_bounds__(DNT) k_desc(const int64_t *__restrict__ h_rp, 
         }
         __shared__ double s_mn[DNT / 32], s_mx[DNT / 32];
         if ((tid & 31) == 0) s_mn[tid >> 5] = mn, s_mx[tid >> 5] = mx;
-        __syncthreads();
-        if (tid == 0) {
-            for (int w = 1; w < DNT / 32; ++w) s_mn[0] = fmin(s_mn[0], s_mn[w]), s_mx[0] = fmax(s_mx[0], s_mx[w]);
-        }
-        __syncthreads();
-        const double gmin = s_mn[0], gmax = s_mx[0];
+        cta_sums(st, scratch);
+        const double dmean = st[0] / nrows, dvar = st[1] / nrows - dmean * dmean, hjj = st[2], hrow = st[3], srow = st[4];
+        const int dmax_reached = s_max;
+        for (int l = tid; l < nat; l += DNT)
+            if (dist[l] == dmax_reached) atomicAdd(&s_surf, 1);
         // --- mean Frobenius norm of the in-subspace neighbour blocks of atom a
-        double fsum = 0.0, fcnt = 0.0;
+        double fs[2] = {0, 0};
         for (int s = tid; s < cnt[la]; s += DNT) {
             const int lc = nbl[la * dmax + s];
             if (lc == la) continue;
             const int64_t kb = nbk[la * dmax + s];
             double f = 0.0;
             for (int q = 0; q < B * B; ++q) f += h_val[kb * B * B + q] * h_val[kb * B * B + q];
-            fsum += sqrt(f);
-            fcnt += 1.0;
+            fs[0] += sqrt(f);
+            fs[1] += 1.0;
         }
-        fsum = cta_sum_d(fsum, scratch);
-        fcnt = cta_sum_d(fcnt, scratch);
-        // --- spectral moments
+        // --- spectral moments; v_k is zero beyond k hops, so step k takes the rows up to
+        // k + 1 hops away and the neighbours up to k (under half of the FP64 products)
         for (int l = tid; l < nrows; l += DNT) v0[l] = (l == jl) ? 1.0 : 0.0;
-        __syncthreads();
+        cta_sums(fs, scratch);
+        const double fsum = fs[0], fcnt = fs[1];
         double mom[10];
         double *cur = v0, *nxt = v1;
         for (int k = 0; k < 5; ++k) {
-            double d1 = 0.0, d2 = 0.0;
+            double d[2] = {0, 0};
+            const int reach = k < 4 ? k + 1 : k; // the last vector is only needed where v_4 is not zero
             for (int l = tid; l < nrows; l += DNT) {
-                const int lat = l / B, i = l % B;
-                double y = -hjj * cur[l];
-                for (int s = 0; s < cnt[lat]; ++s) {
-                    const int lc = nbl[lat * dmax + s];
-                    const int64_t kb = nbk[lat * dmax + s];
-                    for (int q = 0; q < B; ++q) y = fma(h_val[kb * B * B + i * B + q], cur[lc * B + q], y);
+                const int lat = l / B, i = l - lat * B;
+                double y = 0.0;
+                if (dist[lat] <= reach) {
+                    const double x = cur[l];
+                    y = -hjj * x;
+                    for (int s = 0; s < cnt[lat]; ++s) {
+                        const int lc = nbl[lat * dmax + s];
+                        if (dist[lc] > k) continue;
+                        y = dot_row<B>(h_val + (int64_t)nbk[lat * dmax + s] * B * B + i * B, cur + lc * B, y);
+                    }
+                    d[0] += x * x;
+                    d[1] += x * y;
                 }
                 nxt[l] = y;
-                d1 += cur[l] * cur[l];
-                d2 += cur[l] * y;
             }
             // v_k . v_k = m_{2k},  v_k . v_{k+1} = m_{2k+1}
-            mom[2 * k] = cta_sum_d(d1, scratch);
-            mom[2 * k + 1] = cta_sum_d(d2, scratch);
+            cta_sums(d, scratch);
+            mom[2 * k] = d[0];
+            mom[2 * k + 1] = d[1];
             double *t = cur;
             cur = nxt;
             nxt = t;
@@ -215,7 +221,7 @@ __global__ void __launch_bounds__(DNT) k_desc(const int64_t *__restrict__ h_rp, 
             for (int q = 0; q < NDESC; ++q) o[q] = 0.f;
             o[0] = (float)(R / 5.0);
             o[1] = (float)(log((double)nat) / log(1000.0));
-            for (int s = 1; s <= 5; ++s) o[1 + s] = (float)(shells[s] / 100.0);
+            for (int s = 1; s <= 5; ++s) o[1 + s] = (float)(s_shell[s] / 100.0);
             o[7] = (float)((double)(h_rp[j / B + 1] - h_rp[j / B] - 1) / 12.0);
             o[8] = (float)hjj;
             for (int k = 2; k <= 9; ++k) {
@@ -225,12 +231,13 @@ __global__ void __launch_bounds__(DNT) k_desc(const int64_t *__restrict__ h_rp, 
             o[17] = (float)srow;
             o[18] = (float)dmean;
             o[19] = (float)sqrt(fmax(dvar, 0.0));
-            o[20] = (float)gmin;
-            o[21] = (float)gmax;
+            for (int w = 1; w < DNT / 32; ++w) s_mn[0] = fmin(s_mn[0], s_mn[w]), s_mx[0] = fmax(s_mx[0], s_mx[w]);
+            o[20] = (float)s_mn[0];
+            o[21] = (float)s_mx[0];
             o[22] = (float)hrow;
             o[23] = (float)(fcnt > 0 ? fsum / fcnt : 0.0);
             o[24] = (float)(nrows / 1000.0);
-            o[25] = (float)(surf / nat);
+            o[25] = (float)((double)s_surf / nat);
         }
         __syncthreads();
     }

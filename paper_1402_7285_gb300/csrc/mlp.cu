@@ -4,8 +4,8 @@
 // component: this is the project's scheduler model (predicts each column's
 // iterations to tolerance so columns can be ordered / binned).
 //
-// Kernels: per-sample forward (+ backward deltas), per-parameter gradient
-// reduction over the minibatch (a fixed summation order: deterministic), Adam.
+// Kernels: forward (+ backward deltas) per (sample, hidden unit); gradient of the
+// minibatch per parameter (a fixed summation order: deterministic) with the Adam step.
 // Parameter layout (floats): W1[64][32] | b1[64] | W2[64][64] | b2[64] | w3[64] | b3.
 #include <cuda_fp16.h>
 
@@ -19,122 +19,151 @@ namespace {
 constexpr int DI = 32, DH = 64;
 constexpr int O_W1 = 0, O_B1 = O_W1 + DH * DI, O_W2 = O_B1 + DH, O_B2 = O_W2 + DH * DH, O_W3 = O_B2 + DH,
               O_B3 = O_W3 + DH, NPARAM = O_B3 + 1;
-constexpr int FNT = 128;
+constexpr int SPC = 4;        // samples of a CTA
+constexpr int FNT = SPC * DH; // one thread per (sample, hidden unit)
 
-// Forward (and, with T != nullptr, backward deltas) for samples [s0, s0 + n).
+// Forward (and, with DZ1 != nullptr, backward deltas) for samples [s0, s0 + n), one
+// thread per (sample, hidden unit).  A minibatch of 256 samples with one thread per
+// sample kept two SMs busy for 51 us a step (12,000 dependent FMAs a thread); here 64
+// SMs work on it and a thread's chain is 160 FMAs.  W2 has rows of 65 in shared memory:
+// units read it by rows in the forward pass and by columns in the backward pass.
+constexpr int W2LD = DH + 1;
 __global__ void __launch_bounds__(FNT) k_mlp_fwd(const __half *__restrict__ w16, const float *__restrict__ X,
                                                  const float *__restrict__ tgt, int64_t s0, int64_t n,
                                                  float inv_batch, float *__restrict__ pred,
                                                  float *__restrict__ H1, float *__restrict__ H2,
                                                  float *__restrict__ DZ1, float *__restrict__ DZ2,
                                                  float *__restrict__ DY, float *__restrict__ sqerr) {
-    __shared__ float w[NPARAM];
-    for (int i = threadIdx.x; i < NPARAM; i += FNT) w[i] = __half2float(w16[i]);
+    __shared__ float w1[DH * (DI + 1)], w2[DH * W2LD], wr[3 * DH + 1]; // rows padded by one; b1, b2, w3, b3
+    __shared__ float x[SPC][DI], h1[SPC][DH], z2[SPC][DH], err[SPC];
+    for (int i = threadIdx.x; i < NPARAM; i += FNT) {
+        const float v = __half2float(w16[i]);
+        if (i < O_B1) w1[(i / DI) * (DI + 1) + i % DI] = v;
+        else if (i < O_W2) wr[i - O_B1] = v;
+        else if (i < O_B2) w2[((i - O_W2) / DH) * W2LD + (i - O_W2) % DH] = v;
+        else wr[DH + i - O_B2] = v;
+    }
+    const int q = threadIdx.x / DH, u = threadIdx.x % DH;
+    const int64_t t0 = blockIdx.x * (int64_t)SPC, t = t0 + q, s = s0 + t;
+    const bool on = t < n;
+    for (int i = threadIdx.x; i < SPC * DI; i += FNT)
+        x[i / DI][i % DI] = t0 + i / DI < n ? X[(s0 + t0) * DI + i] : 0.f;
     __syncthreads();
-    const int64_t t = blockIdx.x * (int64_t)FNT + threadIdx.x;
+    float acc = wr[u];
+#pragma unroll
+    for (int k = 0; k < DI; ++k) acc = fmaf(w1[u * (DI + 1) + k], x[q][k], acc);
+    const float a1 = tanhf(acc);
+    h1[q][u] = a1;
+    __syncthreads();
+    acc = wr[DH + u];
+#pragma unroll
+    for (int k = 0; k < DH; ++k) acc = fmaf(w2[u * W2LD + k], h1[q][k], acc);
+    const float a2 = tanhf(acc), w3 = wr[2 * DH + u];
+    z2[q][u] = a2;
+    __syncthreads();
+    float y = wr[3 * DH]; // in order, in every thread of the sample
+#pragma unroll
+    for (int i = 0; i < DH; ++i) y = fmaf(wr[2 * DH + i], z2[q][i], y);
+    __syncthreads();
     float err2 = 0.f;
-    if (t < n) {
-        const int64_t s = s0 + t;
-        float x[DI], h1[DH], h2[DH];
+    if (on && pred && u == 0) pred[s] = y;
+    if (tgt) {
+        const float e = on ? y - tgt[s] : 0.f;
+        err2 = e * e;
+        if (DZ1) {
+            const float dy = 2.f * e * inv_batch;
+            const float dz2 = dy * w3 * (1.f - a2 * a2);
+            z2[q][u] = dz2;
+            __syncthreads();
+            acc = 0.f;
 #pragma unroll
-        for (int k = 0; k < DI; ++k) x[k] = X[s * DI + k];
-#pragma unroll 4
-        for (int i = 0; i < DH; ++i) {
-            float acc = w[O_B1 + i];
-#pragma unroll
-            for (int k = 0; k < DI; ++k) acc = fmaf(w[O_W1 + i * DI + k], x[k], acc);
-            h1[i] = tanhf(acc);
-        }
-        float y = w[O_B3];
-#pragma unroll 4
-        for (int i = 0; i < DH; ++i) {
-            float acc = w[O_B2 + i];
-#pragma unroll
-            for (int k = 0; k < DH; ++k) acc = fmaf(w[O_W2 + i * DH + k], h1[k], acc);
-            h2[i] = tanhf(acc);
-            y = fmaf(w[O_W3 + i], h2[i], y);
-        }
-        if (pred) pred[s] = y;
-        if (tgt) {
-            const float e = y - tgt[s];
-            err2 = e * e;
-            if (DZ1) {
-                const float dy = 2.f * e * inv_batch;
-                DY[t] = dy;
-                float dz2[DH];
-#pragma unroll
-                for (int i = 0; i < DH; ++i) {
-                    dz2[i] = dy * w[O_W3 + i] * (1.f - h2[i] * h2[i]);
-                    DZ2[t * DH + i] = dz2[i];
-                    H2[t * DH + i] = h2[i];
-                }
-#pragma unroll 4
-                for (int k = 0; k < DH; ++k) {
-                    float acc = 0.f;
-#pragma unroll
-                    for (int i = 0; i < DH; ++i) acc = fmaf(w[O_W2 + i * DH + k], dz2[i], acc);
-                    DZ1[t * DH + k] = acc * (1.f - h1[k] * h1[k]);
-                    H1[t * DH + k] = h1[k];
-                }
+            for (int i = 0; i < DH; ++i) acc = fmaf(w2[i * W2LD + u], z2[q][i], acc);
+            if (on) {
+                if (u == 0) DY[t] = dy;
+                DZ2[t * DH + u] = dz2;
+                H2[t * DH + u] = a2;
+                DZ1[t * DH + u] = acc * (1.f - a1 * a1);
+                H1[t * DH + u] = a1;
             }
         }
     }
-    if (sqerr) {
-        // per-CTA partial of the squared error (FP64 partials, fixed order)
-        __shared__ float red[FNT];
-        red[threadIdx.x] = err2;
+    if (sqerr) { // per-CTA part of the squared error
+        if (u == 0) err[q] = err2;
         __syncthreads();
-        for (int o = FNT / 2; o > 0; o >>= 1) {
-            if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-            __syncthreads();
+        if (threadIdx.x == 0) {
+            float v = 0.f;
+            for (int k = 0; k < SPC; ++k) v += err[k];
+            sqerr[blockIdx.x] = v;
         }
-        if (threadIdx.x == 0) sqerr[blockIdx.x] = red[0];
     }
 }
 
-// grad[p] = sum over the n samples of the batch, one thread per parameter.
-__global__ void k_mlp_wgrad(const float *__restrict__ X, int64_t s0, int64_t n, const float *__restrict__ H1,
-                            const float *__restrict__ H2, const float *__restrict__ DZ1,
-                            const float *__restrict__ DZ2, const float *__restrict__ DY, float *__restrict__ grad) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= NPARAM) return;
+// Gradient of the minibatch and (w != nullptr) the Adam step.  CTA i owns hidden unit
+// i of both layers (rows i of W1 and W2, b1, b2, w3; CTA 0 also b3), a thread a
+// parameter; up to 1024 samples it adds them in order with 32 loads in flight, larger
+// batches are split over 8 groups of threads whose parts are added in order.  (6337
+// threads in 50 CTAs with one load in flight took 17 us a step of 256 samples, with
+// the Adam step a launch of its own.)
+constexpr int WCH = 8, WPC = 128; // groups at most, threads of a group (99 or 100 parameters)
+struct AdamArgs {
+    float *w, *m, *v;
+    __half *w16;
+    float lr, b1, b2, eps, t;
+};
+__device__ __forceinline__ void adam_step(const AdamArgs &A, int p, float gp) {
+    const float mp = A.b1 * A.m[p] + (1.f - A.b1) * gp;
+    const float vp = A.b2 * A.v[p] + (1.f - A.b2) * gp * gp;
+    A.m[p] = mp;
+    A.v[p] = vp;
+    const float mh = mp / (1.f - powf(A.b1, A.t));
+    const float vh = vp / (1.f - powf(A.b2, A.t));
+    const float wp = A.w[p] - A.lr * mh / (sqrtf(vh) + A.eps);
+    A.w[p] = wp;
+    A.w16[p] = __float2half_rn(wp);
+}
+__global__ void __launch_bounds__(WCH *WPC) k_mlp_wgrad(const float *__restrict__ X, int64_t s0, int64_t n,
+                                                        const float *__restrict__ H1, const float *__restrict__ H2,
+                                                        const float *__restrict__ DZ1, const float *__restrict__ DZ2,
+                                                        const float *__restrict__ DY, float *__restrict__ grad,
+                                                        AdamArgs A) {
+    __shared__ float sum[WCH][WPC];
+    const int i = blockIdx.x, c = threadIdx.x % WPC, g = threadIdx.x / WPC;
+    // column c of this unit's parameters: W2[i][c], W1[i][c - 64], b1, b2, w3, b3
+    const float *fa = nullptr, *fb = nullptr; // factors at sample t: fa[t * la], fb[t * lb]
+    int64_t la = DH, lb = DH;
+    int p = -1;
+    if (c < DH) p = O_W2 + i * DH + c, fa = DZ2 + i, fb = H1 + c;
+    else if (c < DH + DI) p = O_W1 + i * DI + c - DH, fa = DZ1 + i, fb = X + s0 * DI + c - DH, lb = DI;
+    else if (c == DH + DI) p = O_B1 + i, fa = DZ1 + i;
+    else if (c == DH + DI + 1) p = O_B2 + i, fa = DZ2 + i;
+    else if (c == DH + DI + 2) p = O_W3 + i, fa = DY, la = 1, fb = H2 + i;
+    else if (c == DH + DI + 3 && i == 0) p = O_B3, fa = DY, la = 1;
+    const int groups = blockDim.x / WPC;
+    const int64_t per = (n + groups - 1) / groups, t0 = g * per, t1 = t0 + per < n ? t0 + per : n;
     float acc = 0.f;
-    if (p < O_B1) {
-        const int i = p / DI, k = p % DI;
-        for (int64_t t = 0; t < n; ++t) acc = fmaf(DZ1[t * DH + i], X[(s0 + t) * DI + k], acc);
-    } else if (p < O_W2) {
-        const int i = p - O_B1;
-        for (int64_t t = 0; t < n; ++t) acc += DZ1[t * DH + i];
-    } else if (p < O_B2) {
-        const int q = p - O_W2, i = q / DH, k = q % DH;
-        for (int64_t t = 0; t < n; ++t) acc = fmaf(DZ2[t * DH + i], H1[t * DH + k], acc);
-    } else if (p < O_W3) {
-        const int i = p - O_B2;
-        for (int64_t t = 0; t < n; ++t) acc += DZ2[t * DH + i];
-    } else if (p < O_B3) {
-        const int k = p - O_W3;
-        for (int64_t t = 0; t < n; ++t) acc = fmaf(DY[t], H2[t * DH + k], acc);
-    } else {
-        for (int64_t t = 0; t < n; ++t) acc += DY[t];
+    constexpr int U = 32; // loads in flight; the additions stay in order
+    int64_t t = t0;
+    if (fa) {
+        for (; t + U <= t1; t += U) {
+            float x[U], y[U];
+#pragma unroll
+            for (int q = 0; q < U; ++q) x[q] = __ldg(fa + (t + q) * la), y[q] = fb ? __ldg(fb + (t + q) * lb) : 1.f;
+#pragma unroll
+            for (int q = 0; q < U; ++q) acc = fmaf(x[q], y[q], acc); // (times 1: a plain sum)
+        }
+        for (; t < t1; ++t) acc = fmaf(fa[t * la], fb ? fb[t * lb] : 1.f, acc);
     }
-    grad[p] = acc;
+    sum[g][c] = acc;
+    __syncthreads();
+    if (g == 0 && p >= 0) {
+        float v = sum[0][c];
+        for (int k = 1; k < groups; ++k) v += sum[k][c];
+        if (grad) grad[p] = v;
+        if (A.w) adam_step(A, p, v);
+    }
 }
 
-__global__ void k_adam(float *__restrict__ w, __half *__restrict__ w16, const float *__restrict__ g,
-                       float *__restrict__ m, float *__restrict__ v, int t, float lr, float b1, float b2, float eps) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= NPARAM) return;
-    const float gp = g[p];
-    const float mp = b1 * m[p] + (1.f - b1) * gp;
-    const float vp = b2 * v[p] + (1.f - b2) * gp * gp;
-    m[p] = mp;
-    v[p] = vp;
-    const float mh = mp / (1.f - powf(b1, (float)t));
-    const float vh = vp / (1.f - powf(b2, (float)t));
-    const float wp = w[p] - lr * mh / (sqrtf(vh) + eps);
-    w[p] = wp;
-    w16[p] = __float2half_rn(wp);
-}
+inline int wgrad_threads(int64_t n) { return n <= 1024 ? WPC : WCH * WPC; }
 
 __global__ void k_to_half(const float *__restrict__ w, __half *__restrict__ w16) {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
@@ -189,15 +218,15 @@ int mlp_grad(tb_ctx *ctx, const float *params, const float *X, const float *y, i
     st.add(grad, 4 * NPARAM, false, true, &dg);
     int rc = st.commit();
     if (rc) return rc;
-    const int64_t nblk = (n + FNT - 1) / FNT;
+    const int64_t nblk = (n + SPC - 1) / SPC;
     MlpWs w;
     rc = mlp_workspace(ctx, n, nblk, w);
     if (rc) return rc;
     k_to_half<<<(NPARAM + 255) / 256, 256, 0, s>>>((const float *)dp, w.w16);
     k_mlp_fwd<<<(int)nblk, FNT, 0, s>>>(w.w16, (const float *)dX, (const float *)dy, 0, n, 1.f / (float)n, nullptr,
                                         w.H1, w.H2, w.DZ1, w.DZ2, w.DY, w.sq);
-    k_mlp_wgrad<<<(NPARAM + 127) / 128, 128, 0, s>>>((const float *)dX, 0, n, w.H1, w.H2, w.DZ1, w.DZ2, w.DY,
-                                                      (float *)dg);
+    k_mlp_wgrad<<<DH, wgrad_threads(n), 0, s>>>((const float *)dX, 0, n, w.H1, w.H2, w.DZ1, w.DZ2, w.DY, (float *)dg,
+                                         AdamArgs{});
     TB_CUDA_TRY(ctx, cudaGetLastError());
     if (loss) {
         std::vector<float> sq(nblk);
@@ -225,35 +254,40 @@ int mlp_train(tb_ctx *ctx, const float *X, const float *y, int64_t n, int32_t ep
     int rc = st.commit();
     if (rc) return rc;
     const int64_t bmax = std::min<int64_t>(batch, n);
-    const int64_t nblk = (n + FNT - 1) / FNT;
+    const int64_t nblk = (n + SPC - 1) / SPC;
     MlpWs w;
-    rc = mlp_workspace(ctx, bmax, nblk, w);
+    // rows of squared-error parts, one per epoch, read back together (64 MB of them at most)
+    const int64_t rows = loss_hist ? std::max<int64_t>(1, std::min<int64_t>(epochs, (16 << 20) / nblk)) : 1;
+    rc = mlp_workspace(ctx, bmax, loss_hist ? nblk * rows : 1, w);
     if (rc) return rc;
     TB_CUDA_TRY(ctx, cudaMemcpyAsync(w.w, dp, 4 * NPARAM, cudaMemcpyDeviceToDevice, s));
     TB_CUDA_TRY(ctx, cudaMemsetAsync(w.m, 0, 4 * NPARAM, s));
     TB_CUDA_TRY(ctx, cudaMemsetAsync(w.v, 0, 4 * NPARAM, s));
     k_to_half<<<(NPARAM + 255) / 256, 256, 0, s>>>(w.w, w.w16);
     int t = 0;
-    std::vector<float> sq(nblk);
+    std::vector<float> sq;
     for (int ep = 0; ep < epochs; ++ep) {
         for (int64_t s0 = 0; s0 < n; s0 += bmax) {
             const int64_t nb = std::min<int64_t>(bmax, n - s0);
-            k_mlp_fwd<<<(int)((nb + FNT - 1) / FNT), FNT, 0, s>>>(w.w16, (const float *)dX, (const float *)dy, s0, nb,
+            k_mlp_fwd<<<(int)((nb + SPC - 1) / SPC), FNT, 0, s>>>(w.w16, (const float *)dX, (const float *)dy, s0, nb,
                                                                  1.f / (float)nb, nullptr, w.H1, w.H2, w.DZ1, w.DZ2,
                                                                  w.DY, nullptr);
-            k_mlp_wgrad<<<(NPARAM + 127) / 128, 128, 0, s>>>((const float *)dX, s0, nb, w.H1, w.H2, w.DZ1, w.DZ2,
-                                                              w.DY, w.g);
             ++t;
-            k_adam<<<(NPARAM + 255) / 256, 256, 0, s>>>(w.w, w.w16, w.g, w.m, w.v, t, lr, 0.9f, 0.999f, 1e-8f);
+            const AdamArgs A{w.w, w.m, w.v, w.w16, lr, 0.9f, 0.999f, 1e-8f, (float)t};
+            k_mlp_wgrad<<<DH, wgrad_threads(nb), 0, s>>>((const float *)dX, s0, nb, w.H1, w.H2, w.DZ1, w.DZ2, w.DY, nullptr, A);
         }
-        if (loss_hist) {
-            k_mlp_fwd<<<(int)nblk, FNT, 0, s>>>(w.w16, (const float *)dX, (const float *)dy, 0, n, 0.f, nullptr,
-                                                nullptr, nullptr, nullptr, nullptr, nullptr, w.sq);
-            TB_CUDA_TRY(ctx, cudaMemcpyAsync(sq.data(), w.sq, 4 * nblk, cudaMemcpyDeviceToHost, s));
-            TB_CUDA_TRY(ctx, cudaStreamSynchronize(s));
+        if (!loss_hist) continue;
+        k_mlp_fwd<<<(int)nblk, FNT, 0, s>>>(w.w16, (const float *)dX, (const float *)dy, 0, n, 0.f, nullptr, nullptr,
+                                            nullptr, nullptr, nullptr, nullptr, w.sq + ep % rows * nblk);
+        if ((ep + 1) % rows && ep + 1 < epochs) continue;
+        const int64_t first = ep / rows * rows, cnt = ep + 1 - first;
+        sq.resize(nblk * cnt);
+        TB_CUDA_TRY(ctx, cudaMemcpyAsync(sq.data(), w.sq, 4 * nblk * cnt, cudaMemcpyDeviceToHost, s));
+        TB_CUDA_TRY(ctx, cudaStreamSynchronize(s));
+        for (int64_t r = 0; r < cnt; ++r) {
             double acc = 0;
-            for (float v : sq) acc += v;
-            loss_hist[ep] = acc / (double)n;
+            for (int64_t q = 0; q < nblk; ++q) acc += sq[r * nblk + q];
+            loss_hist[first + r] = acc / (double)n;
         }
     }
     TB_CUDA_TRY(ctx, cudaMemcpyAsync(dp, w.w, 4 * NPARAM, cudaMemcpyDeviceToDevice, s));
@@ -277,7 +311,7 @@ int mlp_predict(tb_ctx *ctx, const float *params, const float *X, int64_t n, flo
     rc = mlp_workspace(ctx, 1, 1, w);
     if (rc) return rc;
     k_to_half<<<(NPARAM + 255) / 256, 256, 0, s>>>((const float *)dp, w.w16);
-    k_mlp_fwd<<<(int)((n + FNT - 1) / FNT), FNT, 0, s>>>(w.w16, (const float *)dX, nullptr, 0, n, 0.f,
+    k_mlp_fwd<<<(int)((n + SPC - 1) / SPC), FNT, 0, s>>>(w.w16, (const float *)dX, nullptr, 0, n, 0.f,
                                                         (float *)dpred, nullptr, nullptr, nullptr, nullptr, nullptr,
                                                         nullptr);
     TB_CUDA_TRY(ctx, cudaGetLastError());
