@@ -6,7 +6,8 @@
 // vectors live in shared memory; hop distances come from a level-synchronous
 // breadth-first search inside the subspace; the spectral moments
 // m_k = e_j^T (H_OO - H_jj)^k e_j (k = 2..9) from v_{k+1} = (H_OO - H_jj) v_k
-// with m_{2k} = v_k.v_k and m_{2k+1} = v_k.v_{k+1}.
+// with m_{2k} = v_k.v_k and m_{2k+1} = v_k.v_{k+1}.  Bound by the FP64 pipe and the
+// barriers of the sums.
 #include <algorithm>
 #include <vector>
 

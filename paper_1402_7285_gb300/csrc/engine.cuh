@@ -21,6 +21,15 @@
 //   B   rt -= alpha u, ||rt||^2 (S = I: rho, beta: next A), FP32 copy of rt
 //   X   (terms - 1) Chebyshev steps on S c = t               (barrier only)
 //   R   y (+)= sigma c, t = rt - S y, ||t||^2, rho = y^T rt  [again or beta: next A]
+// What bounds the phases (131072 rows x 64 slots, df, 3 CTAs per SM; HBM floors at the
+// measured 6680 GB/s): A 386 us against 125 (the 12 FP32 operations of a df term: issue
+// 62-69 %, the rest register-read stalls; the product alone takes 236); B 89 against 70;
+// X 83 against 42 (each row of x comes from L2 once per referencing block, 8 TB/s); R
+// 320 (df products again); R in FP32 163 against 93.  The graph took 390 (A with two
+// more recurrences), 333, 12 x (87 + 70), 247 + 168 and 74 for rho: 1333 ms a solve of
+// 64 columns at eta 0.5, 685 here.  Small systems are bound by the barriers and their
+// scalar step, 3-8 us a phase: 256 rows x 2 slots FP64 634 -> 120 us an iteration,
+// Anderson 4096 x 32 FP64 81 -> 37.
 // A sweep that does not reduce the residual (bounds that miss part of the spectrum)
 // ends the kernel with fail = 1; the caller then runs the conjugate-gradient path.
 #pragma once

@@ -14,6 +14,10 @@
 //    barriers a sum instead of four;
 //  - 9x9 blocks transposed (the rows of a block are neighbouring lanes, so a value
 //    load touches 4-7 lines instead of 18) and rows of 4x4 blocks in 16-byte loads.
+// Measured (df): fcc b = 4 with overlap, 608 columns of up to 225 atoms, 643 -> 192 ms; b =
+// 9, 152 columns of up to 561 atoms, 445 -> 207 ms, bound by the longest column.  What
+// bounds it: the latency of the block values from L2 (long-scoreboard stalls; b = 9 df
+// values exceed L2), then barriers and the scalar steps between the short products.
 // Vectors that rows gather (r; with S the sweep vectors) are in shared memory, those
 // that only their own row reads (rt, p, u, t) too when they fit, else in a global
 // slice per CTA; as a last resort all are global.

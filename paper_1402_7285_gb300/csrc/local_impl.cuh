@@ -571,7 +571,11 @@ struct LocalLaunch {
             rc = set_error(ctx, TB_ERR_SIZE, "local subspace needs %zu bytes of shared memory (limit %d)", sm, optin);
             return;
         }
-        const void *fn = has_s ? (const void *)k_local<T, B, true> : (const void *)k_local<T, B, false>;
+        // FP64 and df vectors come here only with an overlap whose spectrum is too wide for sweeps (local_engine.cuh)
+        constexpr bool F32 = std::is_same<T, float>::value;
+        const void *fn = (const void *)k_local<T, B, true>;
+        if constexpr (F32)
+            if (!has_s) fn = (const void *)k_local<T, B, false>;
         cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (e != cudaSuccess) {
             rc = set_error(ctx, TB_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
@@ -584,7 +588,7 @@ struct LocalLaunch {
         const int g = std::max(1, std::min<int>(grid, sms * std::max(per_sm, 1)));
         if (has_s)
             k_local<T, B, true><<<g, LNT, sm, stream>>>(a);
-        else
+        else if constexpr (F32)
             k_local<T, B, false><<<g, LNT, sm, stream>>>(a);
         e = cudaGetLastError();
         if (e != cudaSuccess) rc = set_error(ctx, TB_ERR_CUDA, "k_local launch: %s", cudaGetErrorString(e));
