@@ -142,14 +142,18 @@ int tb_build_csr(const tb_system_spec *spec, uint64_t seed, tb_bsr *H, tb_bsr *S
 #define TB_PREC_DF64 2  /* vectors, SpMM and updates in double-float (hi + lo
                            FP32 pairs, ~48 bits) on the FP32 pipes; FP64
                            scalars, projections and reductions as above.  With
-                           S, the inner solve S r = rt is iterative refinement:
-                           the residual t = rt - S y is kept in df, FP32 CG
-                           sweeps solve S c = t (FP32 vectors, FP32 values of S,
-                           two-float dot products) and each sweep's c is added
-                           to y in df, t -= S c with a df product (an FP32 one
-                           once every ||t|| <= 5e4 inner_tol ||rt||, where its
-                           error stays below inner_tol ||rt|| / 20), until
-                           ||t|| <= inner_tol ||rt||                            */
+                           S, the inner solve S r = rt is iterative refinement
+                           (FP64 panels too): the residual t = rt - S y is kept
+                           in the panel's precision, FP32 sweeps solve S c = t
+                           (FP32 vectors, FP32 values of S; a Chebyshev
+                           polynomial on spectral bounds of S that each call
+                           takes from a short Lanczos run, or conjugate
+                           gradients where the spectrum is wide or not
+                           positive) and each sweep's c is added to y, t -= S c
+                           with a product in the panel's precision (an FP32 one
+                           once every ||t|| is so small that its error stays
+                           below inner_tol ||rt|| / 20), until ||t|| <=
+                           inner_tol ||rt||                                     */
 
 /* Y = A X for a real BSR matrix A (n = n_brows*bdim rows) and a complex panel
  * X of ncols columns: X, Y complex double [n][ncols] (row-major, interleaved).
@@ -177,7 +181,8 @@ typedef struct {
                             residual), default 1e-10                              */
     int32_t max_iter;    /* outer iterations, default 100000                        */
     int32_t precision;   /* TB_PREC_FP64 (default), TB_PREC_MIXED or TB_PREC_DF64 */
-    int32_t panel_w;     /* columns solved together; 0 = autotuned: with >= 128
+    int32_t panel_w;     /* columns solved together; 0 = 64, or as many as there are
+                            (FP32 panels: the next of 8, 16, 32, 64), autotuned with >= 128
                             columns the library times one iteration of its
                             kernels for each width 8..64 and 2 or 3 CTAs per SM
                             and keeps the fastest per column (cached per shape
@@ -194,7 +199,7 @@ typedef struct {
     void *stream;        /* cudaStream_t to queue work on                         */
     int32_t solver;      /* TB_SOLVER_COCG (default) or TB_SOLVER_QMR                */
     int64_t *stats;      /* optional host array [4]: outer iterations, inner
-                            iterations, and (DF64 with S) refinement passes and
+                            iterations (products of the FP32 sweeps), refinement passes and
                             of those the ones that took S c in FP32 (written
                             before returning)                                     */
 } tb_solve_opts;
@@ -253,19 +258,19 @@ int shifted_cocg_solve(tb_ctx *ctx, const tb_bsr *H, const tb_bsr *S, const doub
                        const tb_solve_opts *opts, double *G, int32_t *iters, double *resid,
                        int32_t *status);
 
-/* Times the kernels of one solver iteration (the Sec. 3 step sequence) for
- * the first panel of the given problem (same arguments and options as
- * shifted_cocg_solve, no outputs).  After the panel is initialised, the
- * sequence  A, B, [IC_A, IC_B], C  (the bracketed pair and C only when
- * S != NULL) is launched `reps` times as ordinary launches on opts->stream,
- * each kernel bracketed by CUDA events (with S, a first inner pair runs
- * untimed before the timed one, so IC_A/IC_B are timed in their steady
- * state with a previous search direction).  ms[k] (k < 8) receives the average
- * milliseconds per launch of kernel k: 0 A (H product, shifted steps),
- * 1 B (residual update; with S also the S product of the inner start),
- * 2 IC_A (S product of the inner CG), 3 IC_B (inner CG update), 4 C (rho),
- * 5 R (DF64 with S: refinement pass with S c in df), 6 R with S c in FP32;
- * unused entries are 0.  These are the kernels the solve's graph runs. */
+/* Times the parts of a solver iteration (the Sec. 3 step sequence) for the first
+ * panel of the given problem (same arguments and options as shifted_cocg_solve, no
+ * outputs).  FP64 and DF64: `reps` outer iterations of the persistent solver kernel,
+ * whose phases are timed on the device from barrier to barrier.  FP32 panels (and
+ * overlaps that take conjugate gradients): the kernels of one iteration, launched
+ * `reps` times as ordinary launches on opts->stream, each bracketed by CUDA events
+ * (with S, a first inner pair runs untimed before the timed one).  ms[k] (k < 8)
+ * receives the average milliseconds of part k:
+ * 0 A (H product, direction and shifted steps), 1 B (residual update),
+ * 2 S product of the inner solve (a Chebyshev step, or the product of an inner CG
+ * step), 3 inner CG update, 4 C (rho) (both only where kernels are timed),
+ * 5 R (refinement pass with S c in the panel's precision), 6 R with S c in FP32,
+ * 7 a whole outer iteration (persistent kernel); unused entries are 0. */
 int shifted_cocg_profile(tb_ctx *ctx, const tb_bsr *H, const tb_bsr *S, const double *z, int32_t n_z,
                          const int64_t *rhs_rows, int64_t n_rhs, const int64_t *out_row_ptr,
                          const int64_t *out_rows, const tb_solve_opts *opts, int32_t reps, double *ms);
@@ -288,9 +293,10 @@ int tb_local_subspaces(const tb_bsr *A, const int64_t *rhs_rows, const int32_t *
  * outside O_c give 0).  S (NULL = I) must have H's block pattern.  `order`
  * (optional, a permutation of 0..n_rhs-1) is the order in which columns are
  * taken from the device work queue: each CTA solves one column at a time in
- * shared memory and takes the next as soon as it finishes.  When the vectors
- * of the largest subspace do not fit one CTA's shared memory they are placed
- * in a device workspace of (grid x vectors) instead (read through L2).
+ * shared memory and takes the next as soon as it finishes.  Vectors of the
+ * largest subspace that do not fit a CTA's shared memory, or that leave room for
+ * more CTAs when they are elsewhere, are placed in a device workspace of (grid x
+ * vectors) instead (read through L2).
  * opts->panel_w is ignored; n_z <= 1024.  Outputs and status as
  * shifted_cocg_solve.  TB_ERR_SIZE when even the per-shift states and the
  * local block structure do not fit shared memory. */
