@@ -130,7 +130,7 @@ def measured_peaks() -> dict:
 def kernel_source_hash() -> str:
     """sha256 over the sources of the solver kernels (the ncu figures are valid for these)."""
     h = hashlib.sha256()
-    for f in ("cocg_impl.cuh", "cocg_kernels.cuh", "spmm.cuh", "df64.cuh", "common.cuh"):
+    for f in ("engine.cuh", "cocg_impl.cuh", "cocg_kernels.cuh", "df64.cuh", "common.cuh"):
         h.update(open(os.path.join(ROOT, "paper_1402_7285_gb300", "csrc", f), "rb").read())
     return h.hexdigest()
 
@@ -179,6 +179,26 @@ def algorithmic_bytes(n_rows, nnzb, bdim, n_brows, W, n_z, n_ent, esz, dsz, refi
         out["R_refine"] = 4 * V + 2 * V32 + Mb          # Y, T rw (df); C32 in, T32 out; df S
         out["R_refine_fp32"] = 4 * V + 2 * V32 + Mb32   # the same with S c from FP32 values of S
     return out
+
+
+def phase_bytes(n_rows, nnzb, bdim, n_brows, W, n_z, n_ent, steps, refine_per_outer):
+    """Bytes each phase of the persistent solver (FP64 and df panels with S) must move
+    once: the counterpart of algorithmic_bytes for csrc/engine.cuh.  steps: products
+    of a Chebyshev sweep; the first reads the residual alone and the second needs no
+    x_{k-1}.  The kept rows' p^m and x^m are read and written in one step per
+    outer iteration, spread here over all of them."""
+    V, V32 = n_rows * W * 16, n_rows * W * 8
+    idx = nnzb * 4 + (n_brows + 1) * 8
+    Mb, Mb32 = nnzb * bdim * bdim * 8 + idx, nnzb * bdim * bdim * 4 + idx
+    proj = n_ent * n_z * 16
+    return {
+        "A_outer_H_product": 6 * V + Mb,                             # r, rt, p, u in; p, u out; H
+        "B_update": 3 * V + V32,                                     # rt, u in; rt, FP32 rt out
+        "IC_A_inner_S_product": (4 * steps - 3) / steps * V32 + Mb32 + 4 * proj / (steps * refine_per_outer),
+        "IC_B_inner_update": 0, "C_rho": 0,                          # (kernels of the graph path)
+        "R_refine": 3 * V + 2 * V32 + Mb,                            # rt, c in; r, t, FP32 t out; S
+        "R_refine_fp32": 3 * V + 3 * V32 + Mb32,                     # r rw, rt, c, FP32 t rw; FP32 S
+    }
 
 
 # FP32 instructions per df operation as implemented (csrc/df64.cuh): a lazily
@@ -357,16 +377,23 @@ def run_ours(args, rank, world):
         M = Hh.n_rows
         full_rows = torch.arange(M, device=dev, dtype=torch.int64).repeat(W)
         full_ptr = torch.arange(W + 1, device=dev, dtype=torch.int64) * M
-        base = tb.profile(ctx, H, S, zt, cols, ptr, orows, reps=args.profile_reps, precision=prec, panel_w=W)
-        full = tb.profile(ctx, H, S, zt, cols, full_ptr, full_rows, reps=args.profile_reps, precision=prec,
-                          panel_w=W)
-        torch.cuda.synchronize()
+
+        def ms_per_iteration(p, o):
+            ms = []
+            for n in (2, 2, 2 + args.profile_reps):   # the first call warms up; the difference of the others
+                torch.cuda.synchronize()
+                t0 = time.perf_counter()
+                tb.solve(ctx, H, S, zt, cols, p, o, tol=1e-300, max_iter=n, precision=prec, panel_w=W)
+                torch.cuda.synchronize()
+                ms.append((time.perf_counter() - t0) * 1e3)
+            return (ms[2] - ms[1]) / args.profile_reps
+
+        base, full = ms_per_iteration(ptr, orows), ms_per_iteration(full_ptr, full_rows)
         ctx.close()
-        extra = (full["A_outer_H_product"] + full["B_update"]) - (base["A_outer_H_product"] + base["B_update"])
+        extra = full - base
         nbytes = 5 * W * M * n_z * 16
         return {"full_vector": {"kept_rows_per_column": M, "projection_bytes": 2 * W * M * n_z * 16,
-                                "ms_A_B_block_pattern": base["A_outer_H_product"] + base["B_update"],
-                                "ms_A_B_full_vectors": full["A_outer_H_product"] + full["B_update"],
+                                "ms_iteration_block_pattern": base, "ms_iteration_full_vectors": full,
                                 "pair_step_bytes_per_iteration": nbytes, "pair_step_ms": extra,
                                 "pair_step_gbs": nbytes / (extra * 1e-3) / 1e9,
                                 "frac_of_hbm": nbytes / (extra * 1e-3) / 1e9 / measured_peaks()["hbm_gbs"]}}
@@ -415,10 +442,12 @@ def run_ours(args, rank, world):
     # loop executions x slots against the iterations the columns needed: the work a
     # panel spends on slots that wait for the queue's last columns
     padded_work = (outer * W - col_iters) / max(col_iters, 1)
-    # per panel: 13 set-up and write-out launches, A, B and C per outer iteration,
-    # IC_A and IC_B per inner step and (df64 refinement) one R per inner step
-    refine_mode = prec == tb.TB_PREC_DF64
-    launches = sum(13 + 3 * r.outer_iters + (3 if refine_mode else 2) * r.inner_iters for r in results)
+    # FP64 and df: a solve is one persistent kernel behind two structure checks, the
+    # unit-diagonal check, the spectral bounds, three value conversions and the copy of
+    # z, and the reduction three more.  FP32: 13 set-up and write-out launches, A, B and
+    # C per outer iteration and IC_A, IC_B per inner step
+    persistent = prec != tb.TB_PREC_MIXED
+    launches = sum(12 if persistent else 13 + 3 * r.outer_iters + 2 * r.inner_iters for r in results)
     accuracy = golden_accuracy(results[0], panels[0]) if rank == 0 else None
     ms_max, pairs_all, launches_all = sharding.reduce_step_stats(ms, float(pairs), float(launches), world, dev)
     value = pairs_all / (ms_max / 1e3)
@@ -482,14 +511,18 @@ def run_ours(args, rank, world):
     prof = tb.profile(ctx, H, S, zt, cols, ptr, orows, reps=args.profile_reps, precision=prec, panel_w=W,
                       ctas_per_sm=args.ctas_per_sm)
     counts = {"A_outer_H_product": outer, "B_update": outer, "IC_A_inner_S_product": inner,
-              "IC_B_inner_update": inner, "C_rho": outer, "R_refine": refines - light,
-              "R_refine_fp32": light}
+              "IC_B_inner_update": 0 if persistent else inner, "C_rho": 0 if persistent else outer,
+              "R_refine": refines - light, "R_refine_fp32": light}   # (of the persistent kernel: phases)
     share = {k: prof[k] * counts[k] for k in prof if prof[k] > 0}
     dom = max(share, key=share.get)
     n_ent = int(ptr[-1].item())
     esz = 4 if prec == tb.TB_PREC_MIXED else 8      # bytes per real: FP32, or FP64 / df pairs
     dsz = 4 if prec != tb.TB_PREC_FP64 else 8       # inner CG directions: FP32 with df panels
-    algo = algorithmic_bytes(Hh.n_rows, Hh.nnzb, Hh.bdim, Hh.n_brows, W, n_z, n_ent, esz, dsz, refine=refine_mode)
+    if persistent:
+        algo = phase_bytes(Hh.n_rows, Hh.nnzb, Hh.bdim, Hh.n_brows, W, n_z, n_ent, inner / max(refines, 1),
+                           max(refines, 1) / max(outer, 1))
+    else:
+        algo = algorithmic_bytes(Hh.n_rows, Hh.nnzb, Hh.bdim, Hh.n_brows, W, n_z, n_ent, esz, dsz)
     peaks = measured_peaks()
     achieved = algo[dom] / (prof[dom] * 1e-3) / 1e9
     # the metric's roofline: algorithmic bytes of the dominant kernel per launch / its
