@@ -243,6 +243,10 @@ void tb_solve_opts_default(tb_solve_opts *opts);
  * every diagonal block of S is the identity (orthonormal orbitals on each
  * site; checked on the device per call) the S products add those blocks'
  * operand instead of multiplying by them, with the same result bits.
+ * A column whose stored residual falls below 2^-20 (FP64: 2^-200) is multiplied by a
+ * power of two, and the pi of its shifts with it, so that a seed that converges
+ * long before another shift does not leave the exponents of its vectors; nothing is
+ * rounded by that.
  * TB_PREC_DF64 restart: once a column's seed residual ||S r|| is below 1e-10,
  * its worst unconverged shift residual is checked every 512 outer
  * iterations; if it fell by less than 1 % since the previous check, the

@@ -268,9 +268,11 @@ __device__ __forceinline__ bool pair_coef_B(const Panel<T> &p, int q, c64 &as) {
     as = mk(0.0, 0.0);
     ColState &C = p.col[q / p.nz];
     ShiftState &S = p.sh[q];
-    const c64 sig = p.z[q % p.nz] - C.zs, al = C.alpha, boa = C.boa, pi = S.pi, pi_prev = S.pi_prev;
-    const int done = C.done, active = S.active;
+    const c64 sig = p.z[q % p.nz] - C.zs, al = C.alpha, boa = C.boa;
+    const int step = C.step, done = C.done, active = S.active;
+    const c64 pi = mul_pow2(step, S.pi), pi_prev = mul_pow2(step, S.pi_prev); // as the rows of this phase scale rt
     if (done || !active) return false;
+    if (step) S.pi = pi;
     const c64 pn = (mk(1.0, 0.0) + al * sig) * pi + (al * boa) * (pi - pi_prev);
     const c64 ipn = cinv(pn);
     as = (pi * ipn) * al;
@@ -505,9 +507,9 @@ __device__ bool finish_alpha(const Panel<T> &p, int W, const double *red, ColSta
         const int KM = p.max_col_ent;
         for (int c = threadIdx.x; c < W; c += NT) {
             ColState &C = col[c];
-            const double rn2 = C.rn2;
+            const bool low = below_stall(C.rn2, C.ex, p.stall2);
             const int done = C.done, restarts = C.restarts, chk = C.chk_n, its = C.iters;
-            if (done || !(rn2 < p.stall2) || restarts >= 2) continue;
+            if (done || !low || restarts >= 2) continue;
             if (chk >= 0 && its - chk < 512) continue;
             double rw = -1.0;
             int mw = -1;
@@ -538,6 +540,18 @@ __device__ bool finish_alpha(const Panel<T> &p, int W, const double *red, ColSta
             }
         }
     }
+    // what this iteration's B scales by (a restarting column's rt becomes e_j)
+    for (int c = threadIdx.x; c < W; c += NT) {
+        ColState &C = col[c];
+        C.step = C.done || C.restart ? 0 : range_step<T>(C.rn2);
+        if (C.restart) C.ex = 0;
+        if (C.step) {
+            const double f2 = pow2d(2 * C.step);
+            C.ex += C.step;
+            C.rn2 *= f2; // of the vectors as B will leave them
+            C.rho = f2 * C.rho;
+        }
+    }
     __syncthreads();
     const int all = __syncthreads_and(threadIdx.x < W ? col[threadIdx.x].done != 0 : 1);
     if (threadIdx.x == 0) p.ctl->panel_done = all;
@@ -566,7 +580,7 @@ __global__ void __launch_bounds__(NT, (B <= 4 ? 3 : 1)) k_outer(Panel<T> p) {
 #pragma unroll
     for (int cc = 0; cc < CPT; ++cc) {
         const ColState &C = p.col[lane * CPT + cc];
-        ld.s[cc] = C.done ? mk<T>(0, 0) : cvt<T>(C.beta_prev);
+        ld.s[cc] = C.done ? mk<T>(0, 0) : cvt<T>(C.beta_vec);
     }
     cpx<T> zs[CPT]; // each column's seed shift
 #pragma unroll
@@ -643,7 +657,7 @@ __device__ void finish_outer(const Panel<T> &p, int W, const double *rho_next, i
             continue;
         }
         if (restart) { // first iteration of the new seed follows
-            C.beta_prev = C.boa = mk(0.0, 0.0);
+            C.beta_prev = C.beta_vec = C.boa = mk(0.0, 0.0);
             C.rho = rn;
             C.restart = 0;
             C.fresh = 0;
@@ -652,6 +666,7 @@ __device__ void finish_outer(const Panel<T> &p, int W, const double *rho_next, i
         }
         const c64 be = rn * cinv(rho);
         C.beta_prev = be;
+        C.beta_vec = C.step ? pow2d(C.step) * be : be; // p and u were left as they were
         C.boa = be * cinv(alpha);
         C.rho = rn;
         C.iters = its + 1;
@@ -676,11 +691,13 @@ __global__ void __launch_bounds__(NT, (B <= 4 ? 3 : 1)) k_update_sI(Panel<T> p) 
     constexpr int CPT = TM::CPT;
     const int team = threadIdx.x / TM::TPR, lane = threadIdx.x % TM::TPR;
     cpx<T> a[CPT];
+    int step[CPT];
     unsigned rst = 0; // bit cc: column lane*CPT+cc restarts now (its rt becomes e_j)
 #pragma unroll
     for (int cc = 0; cc < CPT; ++cc) {
         const ColState &C = p.col[lane * CPT + cc];
-        a[cc] = cvt<T>(C.alpha);
+        step[cc] = C.step;
+        a[cc] = cvt<T>(pow2d(step[cc]) * C.alpha);
         rst |= (C.restart ? 1u : 0u) << cc;
     }
     Acc<T> acc[CPT][3];
@@ -700,7 +717,7 @@ __global__ void __launch_bounds__(NT, (B <= 4 ? 3 : 1)) k_update_sI(Panel<T> p) 
                     rt[cc] = mk<T>(row == p.col[lane * CPT + cc].row ? (T)1 : (T)0, 0);
                     clear_restart_row(p, W, p.ctl->n, row, lane * CPT + cc);
                 } else {
-                    rt[cc] = rt[cc] - a[cc] * u[cc];
+                    rt[cc] = mul_pow2(step[cc], rt[cc]) - a[cc] * u[cc];
                 }
                 const T rr = rt[cc].re * rt[cc].re, ii = rt[cc].im * rt[cc].im;
                 acc[cc][0].add(rr);
@@ -737,11 +754,14 @@ __global__ void __launch_bounds__(NT, (B <= 4 ? 3 : 1)) k_update_S(Panel<T> p) {
     const int n = p.ctl->n;
     const T *Rc = p.R[n & 1];
     T *Rn = p.R[(n + 1) & 1];
-    LdGuess<T, W> ld; // y_0 = r_n - alpha_n u
+    // y_0 = r_n - alpha_n u; where rt is scaled (range_step) y_0 is not: it is smaller by
+    // the factor, so that this inner solve starts from next to nothing
+    LdGuess<T, W> ld;
     ld.r = Rc;
     ld.u = p.U;
     ld.lane = lane;
     cpx<T> a[CPT];
+    int step[CPT];
     unsigned rst = 0; // bit cc: column lane*CPT+cc restarts now (its rt becomes e_j)
     // refinement: the first FP32 sweep sees t_0 / ||rt_n|| (no FP32 underflow however
     // small the residuals of a tight solve become); a restarting column's residual
@@ -751,7 +771,8 @@ __global__ void __launch_bounds__(NT, (B <= 4 ? 3 : 1)) k_update_S(Panel<T> p) {
     for (int cc = 0; cc < CPT; ++cc) {
         const ColState &C = p.col[lane * CPT + cc];
         const c64 al = C.alpha;
-        a[cc] = cvt<T>(al);
+        step[cc] = C.step;
+        a[cc] = cvt<T>(pow2d(step[cc]) * al);
         ld.s[cc] = mk((X)(-al.re), (X)(-al.im));
         ld.fresh_row[cc] = C.fresh ? C.row : -1;
         rst |= (C.restart ? 1u : 0u) << cc;
@@ -779,7 +800,7 @@ __global__ void __launch_bounds__(NT, (B <= 4 ? 3 : 1)) k_update_S(Panel<T> p) {
                     rt[cc] = mk<T>(row == p.col[lane * CPT + cc].row ? (T)1 : (T)0, 0);
                     clear_restart_row(p, W, n, row, lane * CPT + cc);
                 } else {
-                    rt[cc] = rt[cc] - a[cc] * u[cc];
+                    rt[cc] = mul_pow2(step[cc], rt[cc]) - a[cc] * u[cc];
                 }
                 t[cc] = rt[cc] - sy[i][cc];
                 acc[cc][0].add(rt[cc].re * rt[cc].re);

@@ -34,7 +34,6 @@ struct ColState {
     c64 alpha;      // alpha_n (0 when the column is done)
     c64 beta_prev;  // beta_{n-1}
     c64 boa;        // beta_{n-1} / alpha_{n-1}
-    c64 rho_next;   // rho_{n+1} (between B/C row work and finalize)
     double rn2;     // ||rt_n||^2
     double in_rr;   // inner CG: t^H t
     double in_alpha, in_beta, in_tol2;
@@ -54,15 +53,48 @@ struct ColState {
     int32_t in_sweep;   // 1 while this column's inner solve is still refining
     int32_t in_conv;    // 1 once ||t|| <= inner_tol ||rt|| (or the refinement cap is reached)
     int32_t in_refines; // refinements made in this outer iteration
-    int32_t pad_;
+    int32_t ex;         // the stored rt, r, p, u and pi are 2^ex times the column's own
     double in_t2;       // ||t||^2 of the true residual at the last refinement
     double in_sig;      // scale of the current FP32 sweep: it solves S c' = t / in_sig
+    // range of the stored vectors (see range_step)
+    c64 beta_vec;       // beta_{n-1} 2^step of B(n-1): the factor of the stored p and u in A(n)
+    int32_t step, pad_[3]; // B(n) multiplies rt_n by 2^step (33 doublewords: slots lie in different banks)
 };
 
 // A residual norm usable as a scale (1 when it is zero or not finite).
 __host__ __device__ __forceinline__ double safe_scale(double norm2) {
     return (norm2 > 1e-300 && norm2 < 1e300) ? sqrt(norm2) : 1.0;
 }
+
+// Range.  COCG is linear in (rt, r, p, u): multiplied by one factor they give the same
+// alpha and beta, and with the pi of all shifts multiplied by it too the same r / pi, so
+// the shifted solutions, residuals and QMR weights do not change either.  The factor is a
+// power of two: nothing is rounded.  df and FP32 vectors have FP32's exponents, and a seed
+// that converges long before another shift (one between two bands, or outside the
+// spectrum) reaches ||rt|| below 1e-19, where the products of the dots underflow: rho_n
+// becomes zero (a breakdown), or ||rt||^2 = 0 passes every shift's residual test.  So a
+// column whose stored norm falls below 2^-20 is brought back to a norm in [1, 2); FP64,
+// whose squares underflow below 1e-154, at 2^-200.
+// Exponents are read and set as integers: an FP64 instruction takes 19 cycles of the
+// chain that every other CTA waits for.
+template <typename T>
+constexpr int range_low() { return std::is_same<T, double>::value ? -400 : -40; } // log2 of the bound's square
+// 2^k (|k| <= 1022)
+__device__ __forceinline__ double pow2d(int k) { return __hiloint2double((1023 + k) << 20, 0); }
+// k > 0: multiply by 2^k a column whose stored vectors have ||rt||^2 = rn2; 0: leave them
+// (in range, or a norm that is zero, subnormal or not finite)
+template <typename T>
+__device__ __forceinline__ int range_step(double rn2) {
+    const int e = (__double2hiint(rn2) >> 20) - 1023; // (rn2 >= 0, or NaN: a large or negative exponent)
+    if (e >= range_low<T>() || e <= -1023) return 0;
+    return (1 - e) / 2; // 2^e <= rn2 < 2^(e + 1), |k| <= 511
+}
+// ||rt||^2 of the column itself below the bound of the stall test (0: never)
+__device__ __forceinline__ bool below_stall(double rn2, int ex, double stall2) {
+    return stall2 > 0.0 && (ex ? (ex > 500 || rn2 * pow2d(-2 * ex) < stall2) : rn2 < stall2);
+}
+
+static_assert(sizeof(ColState) / 8 % 2 == 1, "a thread a slot: no bank conflicts");
 
 struct ShiftState {
     c64 pi, pi_prev, pi_next; // pi_{n-1}, pi_{n-2}, pi_n at the start of A(n)

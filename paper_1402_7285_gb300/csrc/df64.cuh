@@ -132,6 +132,23 @@ __host__ __device__ __forceinline__ df fma_f(df a, float b, df c) {
     return df_fast_two_sum(s.hi, DF_ADD(s.lo, DF_ADD(e, c.lo)));
 }
 
+// z 2^k (exact; df and FP32 values: k <= 127)
+__device__ __forceinline__ cpx<df> mul_pow2(int k, cpx<df> z) {
+    const float f = __uint_as_float((127u + k) << 23);
+    return mk(df(f * z.re.hi, f * z.re.lo), df(f * z.im.hi, f * z.im.lo));
+}
+__device__ __forceinline__ cpx<float> mul_pow2(int k, cpx<float> z) {
+    const float f = __uint_as_float((127u + k) << 23);
+    return mk(DF_MUL(f, z.re), DF_MUL(f, z.im)); // (never contracted into an FMA)
+}
+// (on the integer pipe: FP64 instructions behind a predicate that is off still take their
+// turn, 1.2 us of a phase; zeros and subnormal numbers stay, the result has to be in range)
+__device__ __forceinline__ double mul_pow2(int k, double x) {
+    const int h = __double2hiint(x);
+    return __hiloint2double(h & 0x7ff00000 ? h + (k << 20) : h, __double2loint(x));
+}
+__device__ __forceinline__ cpx<double> mul_pow2(int k, cpx<double> z) { return mk(mul_pow2(k, z.re), mul_pow2(k, z.im)); }
+
 __device__ __forceinline__ df ldg_val(const df *p) {
     const float2 v = __ldg(reinterpret_cast<const float2 *>(p));
     return df(v.x, v.y);

@@ -66,6 +66,7 @@ struct SlotScalars {
     T sig;           // scale of the sweep's correction
     typename std::conditional<std::is_same<T, double>::value, double, float>::type
         inv;         // 1 / (scale of the next sweep's residual); FP64 residuals leave FP32's range
+    int32_t step;    // B: rt is multiplied by 2^step (alpha and the next beta hold it where they need it)
     float ratio;     // sig * inv
     int32_t restart; // B: rt becomes e_row
     int64_t row;
@@ -564,6 +565,7 @@ struct EngineRun {
         if (l.c >= 0) {
             const SlotScalars<T> &C = e.sc[l.c];
             const cpx<T> nal = mk(-C.alpha.re, -C.alpha.im);
+            const int step = C.step;
             const bool rst = C.restart != 0;
             const int64_t jrow = C.row;
             const auto inv = C.inv;
@@ -583,7 +585,7 @@ struct EngineRun {
                         rt[i] = mk<T>(row == jrow ? (T)1 : (T)0, 0);
                         clear_restart_row(p, W, n, row, l.c);
                     } else {
-                        rt[i] = cfma(nal, uv[i], rt[i]);
+                        rt[i] = cfma(nal, uv[i], mul_pow2(step, rt[i]));
                     }
                     st1(p.RT, o, rt[i]);
                     const T rr = rt[i].re * rt[i].re, ii = rt[i].im * rt[i].im;
@@ -777,7 +779,7 @@ struct EngineRun {
     // what A needs of the recurrences (behind finish_outer)
     __device__ __forceinline__ void set_outer() {
         for (int c = threadIdx.x; c < W; c += NT) {
-            e.sc[c].beta = cvt<T>(s.col[c].beta_prev);
+            e.sc[c].beta = cvt<T>(s.col[c].beta_vec);
             e.sc[c].zs = cvt<T>(s.col[c].zs);
         }
     }
@@ -895,7 +897,8 @@ struct EngineRun {
                 const bool fin = finish_alpha(p, W, s.red, s.col);
                 for (int c = threadIdx.x; c < W; c += NT) {
                     const ColState &C = s.col[c];
-                    e.sc[c].alpha = cvt<T>(C.alpha);
+                    e.sc[c].alpha = cvt<T>(C.step ? pow2d(C.step) * C.alpha : C.alpha);
+                    e.sc[c].step = C.step;
                     e.sc[c].restart = C.restart;
                     e.sc[c].row = C.row;
                     if constexpr (HAS_S) e.sc[c].inv = 1.0 / (C.restart ? 1.0 : safe_scale(C.rn2));

@@ -100,6 +100,22 @@ __device__ __forceinline__ cpx<T> local_product(int l, const T *__restrict__ val
     return mk(sr.get(), si.get());
 }
 
+// The column times 2^k (see range_step): its vectors and the pi of its shifts.  A call,
+// so that it takes no registers of the iteration.
+template <typename T, bool HAS_S>
+__device__ __noinline__ void scale_column(int k, T *R, T *RT, T *P, T *U, int nrows, ShiftL *shs, int nz) {
+    for (int l = threadIdx.x; l < nrows; l += blockDim.x) {
+        st1(R, l, mul_pow2(k, ld1(R, l)));
+        if constexpr (HAS_S) st1(RT, l, mul_pow2(k, ld1(RT, l)));
+        st1(P, l, mul_pow2(k, ld1(P, l)));
+        st1(U, l, mul_pow2(k, ld1(U, l)));
+    }
+    for (int m = threadIdx.x; m < nz; m += blockDim.x) {
+        shs[m].pi = mul_pow2(k, shs[m].pi);
+        shs[m].pi_next = mul_pow2(k, shs[m].pi_next);
+    }
+}
+
 template <typename T, int B, bool HAS_S>
 __global__ void __launch_bounds__(1024) k_local2(const __grid_constant__ LocalArgs2<T> g) {
     const LocalArgs<T> &a = g.a; // (64 registers: 1024 threads of an SM, in one CTA or several)
@@ -144,6 +160,7 @@ __global__ void __launch_bounds__(1024) k_local2(const __grid_constant__ LocalAr
     __shared__ int s_col, s_jloc, s_nkept, s_nact, s_status, s_stop, s_restart, s_again;
     __shared__ c64 s_alpha, s_boa, s_beta_prev, s_zs; // s_boa: beta_{n-1} / alpha_{n-1}
     __shared__ double s_rn2;
+    __shared__ int s_step;
     __shared__ cpx<T> s_be, s_nal, s_zt; // beta, -alpha, z_s in T
     __shared__ T s_sig;
     __shared__ typename std::conditional<std::is_same<T, double>::value, double, float>::type s_inv;
@@ -151,7 +168,7 @@ __global__ void __launch_bounds__(1024) k_local2(const __grid_constant__ LocalAr
     // scalars that only thread 0 uses
     c64 rho = mk(1.0, 0.0);
     double t2 = 1.0, sig = 1.0, chk_w = 0.0;
-    int chk_n = -1, restarts = 0;
+    int chk_n = -1, restarts = 0, ex = 0; // ex: the stored vectors are 2^ex times the column's own
 
     c64 *xs = a.scratch + (int64_t)blockIdx.x * 2 * a.max_kept * a.nz;
     c64 *ps = xs + (int64_t)a.max_kept * a.nz;
@@ -234,6 +251,7 @@ __global__ void __launch_bounds__(1024) k_local2(const __grid_constant__ LocalAr
             s_beta_prev = s_boa = mk(0.0, 0.0);
             s_be = mk<T>(0, 0);
             s_rn2 = 1.0;
+            s_step = ex = 0;
             t2 = sig = 1.0;
             s_sig = (T)1;
             s_inv = 1;
@@ -399,7 +417,7 @@ __global__ void __launch_bounds__(1024) k_local2(const __grid_constant__ LocalAr
                 const int nact = s_nact;
                 s_nact = 0;
                 s_restart = 0;
-                if (nact > 0 && s_rn2 < a.stall2 && restarts < 2 && (chk_n < 0 || n - chk_n >= 256)) {
+                if (nact > 0 && below_stall(s_rn2, ex, a.stall2) && restarts < 2 && (chk_n < 0 || n - chk_n >= 256)) {
                     int mw = -1;
                     double rw = -1.0;
                     for (int m = 0; m < a.nz; ++m)
@@ -486,6 +504,12 @@ __global__ void __launch_bounds__(1024) k_local2(const __grid_constant__ LocalAr
                 s_be = cvt<T>(be64);
                 s_boa = be64 * cinv(s_alpha);
                 rho = rn;
+                const int k = s_step = range_step<T>(s_rn2); // the vectors and the pi: below
+                if (k) {
+                    ex += k;
+                    s_rn2 *= pow2d(2 * k);
+                    rho = pow2d(2 * k) * rho;
+                }
             };
             if constexpr (HAS_S) {
                 Acc<T> rr[1];
@@ -522,9 +546,13 @@ __global__ void __launch_bounds__(1024) k_local2(const __grid_constant__ LocalAr
                     rr[2].add(y2);
                 }
                 sums(rr, [&](double *v) {
-                    finish(mk(v[0], v[1]));
                     s_rn2 = v[2];
+                    finish(mk(v[0], v[1]));
                 });
+            }
+            if (s_step) {
+                scale_column<T, HAS_S>(s_step, R, RT, P, U, nrows, shs, a.nz);
+                __syncthreads();
             }
         }
         __syncthreads();

@@ -144,6 +144,8 @@ __global__ void __launch_bounds__(LNT) k_local(LocalArgs<T> a) {
     __shared__ double s_rn2, s_in_rr, s_in_alpha, s_in_beta, s_in_tol2;
     __shared__ int s_status, s_stop, s_in_stop, s_restarts, s_restart, s_chk_n;
     __shared__ double s_chk_w;
+    __shared__ int s_step;
+    int ex = 0; // thread 0: the stored vectors are 2^ex times the column's own
     __shared__ c64 s_zs; // this column's seed shift
 
     const int tid = threadIdx.x;
@@ -217,6 +219,7 @@ __global__ void __launch_bounds__(LNT) k_local(LocalArgs<T> a) {
             s_alpha_prev = mk(1.0, 0.0);
             s_beta_prev = mk(0.0, 0.0);
             s_rn2 = 1.0;
+            ex = 0;
             s_status = TB_COL_MAX_ITER;
             s_stop = (jloc < 0);
             if (jloc < 0) s_status = TB_COL_BREAKDOWN;
@@ -360,7 +363,7 @@ __global__ void __launch_bounds__(LNT) k_local(LocalArgs<T> a) {
             // solutions, active ones start again from zero.
             if (tid == 0) {
                 s_restart = 0;
-                if (s_nact > 0 && !s_stop && s_rn2 < a.stall2 && s_restarts < 2 &&
+                if (s_nact > 0 && !s_stop && below_stall(s_rn2, ex, a.stall2) && s_restarts < 2 &&
                     (s_chk_n < 0 || n - s_chk_n >= 256)) {
                     int mw = -1;
                     double rw = -1.0;
@@ -405,6 +408,7 @@ __global__ void __launch_bounds__(LNT) k_local(LocalArgs<T> a) {
                     s_alpha_prev = mk(1.0, 0.0);
                     s_beta_prev = mk(0.0, 0.0);
                     s_rn2 = 1.0;
+                    ex = 0;
                 }
                 __syncthreads();
                 seed_start();
@@ -522,8 +526,29 @@ __global__ void __launch_bounds__(LNT) k_local(LocalArgs<T> a) {
                 s_alpha_prev = s_alpha;
                 s_rho = rn;
                 s_rn2 = red[2];
+                const int k = s_step = range_step<T>(s_rn2);
+                if (k) {
+                    ex += k;
+                    s_rn2 *= pow2d(2 * k);
+                    s_rho = pow2d(2 * k) * s_rho;
+                }
             }
             __syncthreads();
+            if (const int k = s_step) {
+                for (int l = tid; l < nrows; l += LNT) {
+                    RT[l] = mul_pow2(k, RT[l]);
+                    P[l] = mul_pow2(k, P[l]);
+                    if constexpr (HAS_S) {
+                        R[l] = mul_pow2(k, R[l]);
+                        SP[l] = mul_pow2(k, SP[l]);
+                    }
+                }
+                for (int m = tid; m < a.nz; m += LNT) {
+                    shs[m].pi = mul_pow2(k, shs[m].pi);
+                    shs[m].pi_next = mul_pow2(k, shs[m].pi_next);
+                }
+                __syncthreads();
+            }
         }
         // ---- outputs
         for (int q = tid; q < s_nkept * a.nz; q += LNT) a.G[(k0 + q / a.nz) * a.nz + q % a.nz] = xs[q];
