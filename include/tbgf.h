@@ -63,7 +63,9 @@ typedef struct tb_ctx tb_ctx;
 
 /* Create a context bound to the current CUDA device.  It owns the library's
  * device workspace (grown on demand, freed by tb_ctx_destroy).  One context
- * must not be used from two host threads at once. */
+ * must not be used from two host threads at once.  Its calls may use different
+ * streams: a call that shares workspace with work still queued by an earlier one
+ * lets its stream wait for that work. */
 int tb_ctx_create(tb_ctx **out);
 int tb_ctx_destroy(tb_ctx *ctx);
 const char *tb_status_string(int status);

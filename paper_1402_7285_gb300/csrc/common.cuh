@@ -90,6 +90,9 @@ struct tb_ctx {
     int *chk_dev = nullptr;
     volatile int *chk_host = nullptr;
     cudaEvent_t chk_ev = nullptr;
+    // the last work queued on the workspace that calls leave behind them (WS_SPMM_STAGE)
+    cudaEvent_t stage_ev = nullptr;
+    bool stage_used = false;
 };
 
 namespace tbgf {
@@ -113,7 +116,7 @@ int set_error(tb_ctx *ctx, int code, const char *fmt, ...);
 int ws_get(tb_ctx *ctx, int slot, size_t bytes, void **out);
 
 enum WsSlot {
-    WS_SPMM_STAGE = 0,  // staging for tb_bsr_spmm
+    WS_SPMM_STAGE = 0,  // staging of calls that may return before their work is done (see StageOrder)
     WS_SOLVE_VEC = 1,   // panel vectors of the solver
     WS_SOLVE_SMALL = 2, // per-column / per-shift state, partials, control
     WS_SOLVE_PROJ = 3,  // projected solutions
@@ -121,7 +124,28 @@ enum WsSlot {
     WS_STAGE_OUT = 5,   // staged host outputs
     WS_MATRIX32 = 6,    // FP32 copies of matrix values (mixed precision)
     WS_REDUCE = 7,      // gf_reduce staging
-    WS_COUNT = 8
+    WS_LANCZOS = 8,     // vectors of the spectral bounds
+    WS_COUNT = 9
+};
+
+// Calls with device outputs (products, network, reductions) return with work queued that
+// uses WS_SPMM_STAGE (and, products, the word that holds their fault).  The next call
+// may come on another stream: each such call holds a StageOrder while it queues, which
+// lets its stream wait for the last work queued there and marks its own on the way out.
+// (Always, not only when the stream differs: the handle of a destroyed stream can come
+// back.)  Nothing is waited for or marked while the stream is captured.
+class StageOrder {
+  public:
+    StageOrder(tb_ctx *ctx, cudaStream_t s);
+    ~StageOrder();
+    StageOrder(const StageOrder &) = delete;
+    StageOrder &operator=(const StageOrder &) = delete;
+    int rc = TB_OK;
+
+  private:
+    tb_ctx *ctx_;
+    cudaStream_t stream_;
+    bool on_ = false;
 };
 
 bool is_device_ptr(const void *p);
@@ -176,10 +200,12 @@ __device__ __forceinline__ int bsr_row_fault(const int64_t *rp, const int32_t *c
 __global__ void k_validate_bsr(const int64_t *rp, const int32_t *ci, int64_t n_brows, int64_t nnzb, int *bad);
 
 // A checking kernel's result reaches the host without an allocation, a memset or
-// a copy: check_words() gives (once per context) three device words and a pinned
-// host word (of 512 pinned bytes, whose rest serves other small results); the kernel ORs what it finds into words[0] and its last CTA calls
-// publish_check, which writes the result to words[2] (for kernels queued behind
-// it) and to the host word, and clears the others for the next check.
+// a copy: check_words() gives (once per context) four device words and a pinned
+// host word (of 512 pinned bytes, whose rest serves other small results); the kernel ORs
+// what it finds into words[0] and its last CTA calls publish_check, which writes the
+// result to the host word and clears the others for the next check.  A product queued
+// behind its check reads the result from words[2], which no other check writes (its calls
+// are ordered by StageOrder).
 // check_wait() records an event behind the kernel, waits for it and returns the
 // result.  (cudaMallocAsync + memset + copy + cudaFreeAsync with the default
 // pool, which gives its memory back at every synchronisation, took 190 us.)
@@ -220,10 +246,11 @@ __device__ __forceinline__ bool last_cta_arrival(unsigned int *counter) {
 }
 
 // The end of a checking kernel (see check_words): every thread of every CTA calls it.
-__device__ __forceinline__ void publish_check(int *words, int *host) {
+// out: a device word for the result too (null: none).
+__device__ __forceinline__ void publish_check(int *words, int *host, int *out = nullptr) {
     if (last_cta_arrival(reinterpret_cast<unsigned int *>(words + 1)) && threadIdx.x == 0) {
         const int r = atomicExch(words, 0);
-        words[2] = r;
+        if (out) *out = r;
         *reinterpret_cast<volatile int *>(host) = r;
         __threadfence_system();
     }

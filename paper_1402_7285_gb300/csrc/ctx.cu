@@ -47,6 +47,30 @@ int ws_get(tb_ctx *ctx, int slot, size_t bytes, void **out) {
     return TB_OK;
 }
 
+static bool capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) { // the legacy stream during a capture elsewhere
+        cudaGetLastError();
+        return true;
+    }
+    return st != cudaStreamCaptureStatusNone;
+}
+
+StageOrder::StageOrder(tb_ctx *ctx, cudaStream_t s) : ctx_(ctx), stream_(s) {
+    if (capturing(s)) return;
+    cudaError_t e = cudaSuccess;
+    if (!ctx->stage_ev) e = cudaEventCreateWithFlags(&ctx->stage_ev, cudaEventDisableTiming);
+    if (e == cudaSuccess && ctx->stage_used) e = cudaStreamWaitEvent(s, ctx->stage_ev, 0);
+    if (e != cudaSuccess)
+        rc = set_error(ctx, TB_ERR_CUDA, "order of the workspace's calls: %s", cudaGetErrorString(e));
+    else
+        on_ = true;
+}
+
+StageOrder::~StageOrder() {
+    if (on_ && cudaEventRecord(ctx_->stage_ev, stream_) == cudaSuccess) ctx_->stage_used = true;
+}
+
 bool is_device_ptr(const void *p) {
     if (!p) return false;
     cudaPointerAttributes a;
@@ -191,6 +215,7 @@ int tb_ctx_destroy(tb_ctx *ctx) {
         cudaFreeHost((void *)ctx->chk_host);
         cudaEventDestroy(ctx->chk_ev);
     }
+    if (ctx->stage_ev) cudaEventDestroy(ctx->stage_ev);
     if (dev >= 0 && dev != ctx->device) cudaSetDevice(dev);
     delete ctx;
     return TB_OK;

@@ -163,7 +163,7 @@ int spectral_bounds(tb_ctx *ctx, const int64_t *rp, const int32_t *ci, const dou
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((n + NT - 1) / NT, sms));
     const size_t vb = align_up(sizeof(float) * n, 256), pb = align_up(sizeof(double) * 2 * grid, 256);
     void *wsp = nullptr;
-    int rc = ws_get(ctx, WS_SPMM_STAGE, 3 * vb + pb + 4096, &wsp);
+    int rc = ws_get(ctx, WS_LANCZOS, 3 * vb + pb + 4096, &wsp);
     if (rc) return rc;
     char *ws = (char *)wsp;
     int *words = nullptr, *host = nullptr;

@@ -222,6 +222,8 @@ int mlp_grad(tb_ctx *ctx, const float *params, const float *X, const float *y, i
     MlpWs w;
     rc = mlp_workspace(ctx, n, nblk, w);
     if (rc) return rc;
+    StageOrder order(ctx, s);
+    if (order.rc) return order.rc;
     k_to_half<<<(NPARAM + 255) / 256, 256, 0, s>>>((const float *)dp, w.w16);
     k_mlp_fwd<<<(int)nblk, FNT, 0, s>>>(w.w16, (const float *)dX, (const float *)dy, 0, n, 1.f / (float)n, nullptr,
                                         w.H1, w.H2, w.DZ1, w.DZ2, w.DY, w.sq);
@@ -260,6 +262,8 @@ int mlp_train(tb_ctx *ctx, const float *X, const float *y, int64_t n, int32_t ep
     const int64_t rows = loss_hist ? std::max<int64_t>(1, std::min<int64_t>(epochs, (16 << 20) / nblk)) : 1;
     rc = mlp_workspace(ctx, bmax, loss_hist ? nblk * rows : 1, w);
     if (rc) return rc;
+    StageOrder order(ctx, s);
+    if (order.rc) return order.rc;
     TB_CUDA_TRY(ctx, cudaMemcpyAsync(w.w, dp, 4 * NPARAM, cudaMemcpyDeviceToDevice, s));
     TB_CUDA_TRY(ctx, cudaMemsetAsync(w.m, 0, 4 * NPARAM, s));
     TB_CUDA_TRY(ctx, cudaMemsetAsync(w.v, 0, 4 * NPARAM, s));
@@ -310,6 +314,8 @@ int mlp_predict(tb_ctx *ctx, const float *params, const float *X, int64_t n, flo
     MlpWs w;
     rc = mlp_workspace(ctx, 1, 1, w);
     if (rc) return rc;
+    StageOrder order(ctx, s);
+    if (order.rc) return order.rc;
     k_to_half<<<(NPARAM + 255) / 256, 256, 0, s>>>((const float *)dp, w.w16);
     k_mlp_fwd<<<(int)((n + SPC - 1) / SPC), FNT, 0, s>>>(w.w16, (const float *)dX, nullptr, 0, n, 0.f,
                                                         (float *)dpred, nullptr, nullptr, nullptr, nullptr, nullptr,

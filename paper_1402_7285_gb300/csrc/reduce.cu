@@ -129,6 +129,8 @@ extern "C" int gf_reduce_ldos_dm(tb_ctx *ctx, const double *G, int32_t n_z, cons
     void *wsp = nullptr;
     rc = ws_get(ctx, WS_SPMM_STAGE, sizeof(double) * std::max<int64_t>(n_out, 1) + 256, &wsp);
     if (rc) return rc;
+    StageOrder order(ctx, s);
+    if (order.rc) return order.rc;
     double *wt = (double *)wsp;
     int *missing = (int *)((char *)wsp + align_up(sizeof(double) * std::max<int64_t>(n_out, 1), 128));
     const int g = 152 * 4;

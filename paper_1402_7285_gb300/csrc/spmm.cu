@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(SNT) k_spmm_prep(const int64_t *rp, const int3
         convert_span(val, vdst, nval);
         convert_span(X, xdst, nx);
     }
-    publish_check(words, host);
+    publish_check(words, host, words + 2);
 }
 
 // ------------------------------------------------------------------ product
@@ -386,6 +386,8 @@ extern "C" int tb_bsr_spmm(tb_ctx *ctx, const tb_bsr *A, const double *X, int32_
     int *words = nullptr, *host = nullptr, fault = 0;
     rc = check_words(ctx, &words, &host);
     if (rc) return rc;
+    StageOrder order(ctx, s);
+    if (order.rc) return order.rc;
     const int64_t items = std::max<int64_t>(A->n_brows, (f32 || dfp) ? nx / 4 : 0);
     const int g = (int)std::max<int64_t>(1, std::min<int64_t>((items + SNT - 1) / SNT, (int64_t)sm_count() * 8));
     const int64_t nv = A->nnzb * bb;
@@ -458,6 +460,8 @@ extern "C" int tb_bsr_spmm_profile(tb_ctx *ctx, const tb_bsr *A, int32_t ncols, 
     rc = ws_get(ctx, WS_SPMM_STAGE, off_flush + flush_bytes, &wsp);
     if (rc) return rc;
     char *ws = (char *)wsp;
+    StageOrder order(ctx, s);
+    if (order.rc) return order.rc;
     const void *mval = val;
     if (f32 || dfp) {
         convert_values(precision, (const double *)val, ws + off_val, A->nnzb * bb, s);
