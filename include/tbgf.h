@@ -110,7 +110,9 @@ typedef struct {
 /* Block-sparse row matrix with bdim x bdim blocks.
  *   row_ptr int64[n_brows+1], col_idx int32[nnzb] ascending within each block
  *   row with the diagonal block present, val double[nnzb*bdim*bdim] with each
- *   block row-major.  bdim = 1 is plain CSR. */
+ *   block row-major.  bdim = 1 is plain CSR.  val in device memory lies on a
+ *   16-byte boundary (TB_ERR_ARG otherwise; the S of shifted_cocg_solve_local,
+ *   and of reductions and descriptors, on an 8-byte one). */
 typedef struct {
     int64_t n_brows;
     int32_t bdim;

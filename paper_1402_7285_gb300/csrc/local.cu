@@ -258,7 +258,10 @@ extern "C" int shifted_cocg_solve_local(tb_ctx *ctx, const tb_bsr *H, const tb_b
         const size_t o_gvec = la2.own_global ? take((ow + (la2.own_global == 2 ? ga : 0)) * L.grid) : 0;
         const size_t o_zc = take(sizeof(c64) * n_z), o_q = take(sizeof(unsigned long long) * 8);
         const size_t o_h = lowp ? take(sizeof(double) * H->nnzb * bb) : 0;
-        const size_t o_s = lowp && has_s ? take(sizeof(double) * S->nnzb * bb) : 0;
+        // FP64 vectors read S's values as the caller has them, in 16-byte loads: from a copy where they do not lie on
+        // 16-byte boundaries (H's have to, S's never had to)
+        const bool copy_s = !lowp && has_s && ((uintptr_t)d_sval & 15u);
+        const size_t o_s = (lowp && has_s) || copy_s ? take(sizeof(double) * S->nnzb * bb) : 0;
         const size_t o_sf = has_s ? take(sizeof(float) * S->nnzb * bb) : 0;
         void *wsp = nullptr;
         rc = ws_get(ctx, WS_SOLVE_SMALL, off, &wsp);
@@ -275,6 +278,10 @@ extern "C" int shifted_cocg_solve_local(tb_ctx *ctx, const tb_bsr *H, const tb_b
         };
         la.h_val = (const double *)d_hval;
         la.s_val = has_s ? (const double *)d_sval : nullptr;
+        if (copy_s) {
+            TB_CUDA_TRY(ctx, cudaMemcpyAsync(ws + o_s, d_sval, sizeof(double) * nv, cudaMemcpyDeviceToDevice, stream));
+            la.s_val = (const double *)(ws + o_s);
+        }
         if (lowp) {
             convert(TB_PREC_DF64, d_hval, o_h);
             la.h_val = (const double *)(ws + o_h);
