@@ -794,7 +794,8 @@ struct EngineRun {
             double t2 = s.red[3 * c];
             if (mode == 2) t2 *= C.in_sig * C.in_sig;
             const double eta2 = p.inner_tol * p.inner_tol * C.rn2;
-            if (isfinite(t2) && isfinite(C.in_t2) && t2 > 1e-4 * C.in_t2 && t2 > eta2) s.fail = 1;
+            // (written so that a t2 that is not finite, an FP32 sweep that overflowed, fails too)
+            if (isfinite(C.in_t2) && !(t2 <= 1e-4 * C.in_t2) && !(t2 <= eta2)) s.fail = 1;
             C.in_sig = safe_scale(C.in_t2); // the scale the rows used for the next sweep
             C.in_t2 = t2;
             set_sweep(c, C.in_sig, t2);

@@ -340,8 +340,8 @@ __global__ void __launch_bounds__(1024) k_local2(const __grid_constant__ LocalAr
                     ++passes;
                     sums(acc, [&](double *v) {
                         const double eta2 = a.inner_tol * a.inner_tol * s_rn2;
-                        if (isfinite(v[0]) && isfinite(t2) && v[0] > 1e-4 * t2 && v[0] > eta2) {
-                            *g.fail = 1; // the bounds missed part of the spectrum: the caller takes another path
+                        if (isfinite(t2) && !(v[0] <= 1e-4 * t2) && !(v[0] <= eta2)) {
+                            *g.fail = 1; // the bounds missed part of the spectrum (v[0] may not be finite): the caller takes another path
                             s_stop = 1;
                         }
                         sig = safe_scale(t2);
