@@ -1000,7 +1000,8 @@ __global__ void __launch_bounds__(NT, engine_ctas<RPT>()) k_engine(const __grid_
 // a sweep (df) or in all (FP64), or the bounds are not those of a definite matrix.
 template <class E>
 bool chebyshev_terms(double lo, double hi, double inner_tol, int inner_max, bool lowp, E &en) {
-    if (!(lo > 0) || !(hi >= lo) || !std::isfinite(hi) || hi > 30 * lo) return false;
+    // (FP32 holds the values of S and the coefficients, which go with 1 / hi)
+    if (!(lo > 1e-30) || !(hi >= lo) || !(hi < 1e30) || hi > 30 * lo) return false;
     const double theta = 0.5 * (hi + lo), delta = std::max(0.5 * (hi - lo), 1e-3 * theta), s1 = theta / delta;
     const double rate = s1 - std::sqrt(s1 * s1 - 1.0);
     const int passes = std::max(1, (int)std::ceil(std::log(inner_tol) / std::log(3e-7)));

@@ -98,6 +98,7 @@ __global__ void __launch_bounds__(NT, 2) k_lanczos(const __grid_constant__ LzArg
         a.u[1][r] = a.u[2][r] = 0.f;
     }
     float alpha = 0.f, bi_prev = 0.f;
+    double size = 0; // of S: |alpha_0| + beta_1
     for (int k = 0; k < LZ_STEPS; ++k) {
         // t_k = w - alpha_{k-1} v_{k-1} and its norm (t_0: the start vector)
         float *t = a.u[1 + (k & 1)], *tp = a.u[2 - (k & 1)];
@@ -111,7 +112,8 @@ __global__ void __launch_bounds__(NT, 2) k_lanczos(const __grid_constant__ LzArg
         if (!lz_step(a, gen, s0, [&](double t0) { a.ab[2 + 2 * k] = t0 > 0 ? sqrt(t0) : 0; })) return;
         // the scalars of the last CTA: __ldcg, they change while the kernel runs
         const double beta = __ldcg(a.ab + 2 + 2 * k);
-        if (!(beta > 1e-5)) break; // the Krylov space is exhausted
+        if (k == 1) size = fabsf(alpha) + beta;
+        if (!(beta > 1e-5 * size)) break; // the Krylov space is exhausted
         const float bi = (float)(1.0 / beta), bp = (float)beta * bi_prev;
         s0 = 0.f;
         for (int64_t r = tid; r < n; r += stride) {
