@@ -86,6 +86,13 @@ __device__ bool lz_step(const LzArgs &a, unsigned &gen, float s0, F last) {
     return ok != 0;
 }
 
+__device__ void timed_out(const LzArgs &a) {
+    if (threadIdx.x == 0) {
+        *reinterpret_cast<volatile double *>(a.host) = -1.0;
+        __threadfence_system();
+    }
+}
+
 __global__ void __launch_bounds__(NT, 2) k_lanczos(const __grid_constant__ LzArgs a) {
     const int64_t tid = blockIdx.x * (int64_t)NT + threadIdx.x, stride = (int64_t)gridDim.x * NT;
     const int b = a.b;
@@ -109,7 +116,7 @@ __global__ void __launch_bounds__(NT, 2) k_lanczos(const __grid_constant__ LzArg
             t[r] = x;
             s0 += x * x;
         }
-        if (!lz_step(a, gen, s0, [&](double t0) { a.ab[2 + 2 * k] = t0 > 0 ? sqrt(t0) : 0; })) return;
+        if (!lz_step(a, gen, s0, [&](double t0) { a.ab[2 + 2 * k] = t0 > 0 ? sqrt(t0) : 0; })) return timed_out(a);
         // the scalars of the last CTA: __ldcg, they change while the kernel runs
         const double beta = __ldcg(a.ab + 2 + 2 * k);
         if (k == 1) size = fabsf(alpha) + beta;
@@ -133,7 +140,7 @@ __global__ void __launch_bounds__(NT, 2) k_lanczos(const __grid_constant__ LzArg
                 a.ab[0] = k + 1;
                 a.ab[3 + 2 * k] = t0;
             }))
-            return;
+            return timed_out(a);
         alpha = (float)__ldcg(a.ab + 3 + 2 * k);
         bi_prev = bi;
     }
@@ -179,6 +186,7 @@ int spectral_bounds(tb_ctx *ctx, const int64_t *rp, const int32_t *ci, const dou
     a.ab = (double *)(ws + 3 * vb + pb + 3584);
     a.host = (double *)host + 8;
     static_assert(sizeof(GridBarrier) <= 3584, "workspace layout");
+    *(volatile double *)a.host = 0.0; // nothing of an earlier call
     TB_CUDA_TRY(ctx, cudaMemsetAsync(a.bar, 0, 4096, s));
     void *args[] = {&a};
     TB_CUDA_TRY(ctx, cudaLaunchCooperativeKernel((const void *)k_lanczos, dim3(grid), dim3(NT), args, 0, s));
@@ -186,7 +194,8 @@ int spectral_bounds(tb_ctx *ctx, const int64_t *rp, const int32_t *ci, const dou
     rc = check_wait(ctx, s, &dummy);
     if (rc) return rc;
     const volatile double *h = (const volatile double *)host + 8;
-    const int k = (int)h[0];
+    const int k = (int)h[0]; // steps made; -1: a grid barrier timed out
+    TB_CHECK(ctx, k >= 0, TB_ERR_CUDA, "spectral bounds of S: a grid barrier timed out");
     if (k < 1 || k > LZ_STEPS) return TB_OK;
     double d[LZ_STEPS], e[LZ_STEPS], r = 0;
     for (int i = 0; i < k; ++i) {
