@@ -155,8 +155,9 @@ int tb_build_csr(const tb_system_spec *spec, uint64_t seed, tb_bsr *H, tb_bsr *S
                            gradients where the spectrum is wide or not
                            positive) and each sweep's c is added to y, t -= S c
                            with a product in the panel's precision (an FP32 one
-                           once every ||t|| is so small that its error stays
-                           below inner_tol ||rt|| / 20), until ||t|| <=
+                           once every ||t|| is so small, for the spectrum
+                           of S, that its error stays below inner_tol ||rt|| /
+                           20), until ||t|| <=
                            inner_tol ||rt||                                     */
 
 /* Y = A X for a real BSR matrix A (n = n_brows*bdim rows) and a complex panel

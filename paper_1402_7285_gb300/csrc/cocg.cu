@@ -181,7 +181,9 @@ int run_solver(tb_ctx *ctx, const tb_bsr *H, const tb_bsr *S, const double *z, i
         rc = spectral_bounds(ctx, (const int64_t *)d_srp, (const int32_t *)d_sci, (const double *)d_sval, S->n_brows, b,
                              num_sms(), stream, &lo, &hi);
         if (rc) return rc;
-        engine = chebyshev_terms(lo, hi, inner_tol, inner_max, lowp, en);
+        const double light = engine_light(lo, hi);
+        engine = chebyshev_terms(lo, hi, inner_tol, inner_max, lowp, en, lowp ? light : 0.0, &en.terms2);
+        en.light = (float)light;
     }
     // slots: the panel width asked for, or 64 (the graph: the next compiled width up to 32, FP32 64); the persistent
     // kernel takes any number, and then no more than there are columns.  C2 (131072 rows, df64, 64 columns): 64 slots

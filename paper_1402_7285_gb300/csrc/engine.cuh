@@ -39,10 +39,12 @@
 namespace tbgf {
 
 constexpr int MAX_TERMS = 40;
-// A refinement pass takes S c and the residual in FP32 when every residual is below
-// this many inner tolerances: FP32 rounding (below 1e-7 of the residual before the
-// sweep) then stays below inner_tol ||rt|| / 20.
-constexpr double ENGINE_LIGHT = 5e5;
+// A df refinement pass takes S c and the residual in FP32 when every residual is below
+// this many inner tolerances.  The FP32 residual t - S c errs by up to 1.2e-7 sqrt(hi / lo)
+// of the t before the sweep (c is larger along the lowest eigenvectors, where S c cancels;
+// emulated on s-p and s+p+d overlaps: 0.4 to 1.5e-7 at hi / lo = 1.6, 0.6 to 5.6e-7 at 24):
+// below inner_tol ||rt|| / 20.
+inline double engine_light(double lo, double hi) { return 0.05 / (1.2e-7 * std::sqrt(hi / lo)); }
 enum EngineFlag : unsigned { F_CONT = 1, F_AGAIN = 2, F_LIGHT = 4, F_LIST = 8, F_DONE = 16, F_ABORT = 32 };
 enum EnginePhase { PH_A = 0, PH_B = 1, PH_X = 2, PH_R = 5, PH_R32 = 6, PH_INIT = 7 };
 
@@ -79,9 +81,11 @@ struct Engine {
     c64 *kr;            // [W][max_col_ent]: r_n on the kept rows
     GridBarrier *bar;
     int32_t W;        // slots = row stride of the panel
-    int32_t terms;    // Chebyshev terms of a sweep (2..MAX_TERMS)
+    int32_t terms;    // Chebyshev terms of the first sweep of a solve (2..MAX_TERMS)
+    int32_t terms2;   // of the others
     int32_t profile;
     int32_t group;    // CTAs of a group of the two-step sums (at most 64 groups)
+    float light;      // a pass in FP32 below this many inner tolerances (engine_light; 0: never)
     float inv_theta;
     float om[MAX_TERMS], ga[MAX_TERMS]; // x_{k+1} = x_k + om (x_k - x_{k-1}) + ga (b - S x_k)
     float *X[2];
@@ -667,12 +671,12 @@ struct EngineRun {
 
     // ------------------------------------------------------------ refinement pass
     // mode 0: y = sigma c, t = rt - S y (first pass); 1: y += sigma c, t -= S sigma c;
-    // 2: as 1 with S c and the residual in FP32 (the correction is small, see ENGINE_LIGHT).
+    // 2: as 1 with S c and the residual in FP32 (the correction is small, see engine_light).
     // The pass in FP32 for kernels with the rows of a block in a thread: two slots a
     // thread halve the loads of S and of the index arrays.
     __device__ void phase_R32x2() {
         const Layout g = make_layout(W / 2, 2, units);
-        const float *c32 = e.X[e.terms & 1];
+        const float *c32 = e.X[e.terms2 & 1];
         Acc<T> acc[6];
 #pragma unroll
         for (int k = 0; k < 6; ++k) acc[k].zero();
@@ -712,11 +716,12 @@ struct EngineRun {
         }
         engine_partials<T, 3, 2>(acc, g, p.part, s.sp);
     }
+    __device__ __forceinline__ int terms_of(int mode) const { return mode == 0 ? e.terms : e.terms2; }
     __device__ void phase_R(int mode) {
         if constexpr (RPT > 1 && HAS_S) {
             if (mode == 2 && W % 2 == 0) return phase_R32x2();
         }
-        const float *c32 = e.X[e.terms & 1];
+        const float *c32 = e.X[terms_of(mode) & 1];
         Acc<T> acc[3];
         acc[0].zero(), acc[1].zero(), acc[2].zero();
         if (l.c >= 0) {
@@ -802,7 +807,7 @@ struct EngineRun {
             C.in_refines += 1;
             if (t2 > eta2 && isfinite(t2) && C.in_refines < p.refine_max) {
                 s.any = 1;
-                const double lim = ENGINE_LIGHT * p.inner_tol;
+                const double lim = e.light * p.inner_tol;
                 if (!(t2 <= lim * lim * C.rn2)) s.light = 0;
             }
             s.rho[2 * c] = s.red[3 * c + 1];
@@ -810,7 +815,7 @@ struct EngineRun {
         }
         __syncthreads();
         if (threadIdx.x == 0) {
-            p.ctl->inner_total += e.terms - 1;
+            p.ctl->inner_total += terms_of(mode) - 1;
             p.ctl->refine_total += 1;
             p.ctl->light_total += (mode == 2);
             if (s.fail) e.bar->fail = 1;
@@ -833,7 +838,7 @@ struct EngineRun {
     __device__ unsigned inner_solve(int init) {
         int mode = 0;
         for (;;) {
-            for (int k = 1; k < e.terms; ++k) {
+            for (int k = 1; k < terms_of(mode); ++k) {
                 // the kept rows' FP64 updates run beside the first FP32 product
                 if (!init && mode == 0 && k == 1) kept_rows<true, true>();
                 phase_X(k);
@@ -995,24 +1000,44 @@ __global__ void __launch_bounds__(NT, engine_ctas<RPT>()) k_engine(const __grid_
 // ------------------------------------------------------------------ host side
 // Chebyshev coefficients of a sweep for a spectrum within [lo, hi] (x_{k+1} = x_k +
 // om_k (x_k - x_{k-1}) + ga_k (b - S x_k), x_1 = b / theta; Saad, Iterative Methods,
-// Sec. 12.3).  The sweeps of an inner solve share inner_tol evenly, each at best
-// 3e-7 (FP32 rounding); false where they would take more than inner_max products in
-// a sweep (df) or in all (FP64), or the bounds are not those of a definite matrix.
+// Sec. 12.3; the first n of them are those of a sweep of n terms).  The sweeps of an
+// inner solve share inner_tol evenly, each at best 3e-7 (FP32 rounding); false where they
+// would take more than inner_max products in a sweep (df) or in all (FP64), or the bounds
+// are not those of a definite matrix.
+// light > 0 (df panels, engine_light): where the first sweep can end below light inner
+// tolerances, FP32 rounding included, it is given the terms for a quarter of that and the
+// others what is left: the passes behind it then run in FP32.  C2 (hi / lo 1.6): 8 and 6
+// terms, 12 products, as 7 and 7 take, which left the first residual at 5e-7, above light.
 template <class E>
-bool chebyshev_terms(double lo, double hi, double inner_tol, int inner_max, bool lowp, E &en) {
+bool chebyshev_terms(double lo, double hi, double inner_tol, int inner_max, bool lowp, E &en, double light = 0.0,
+                     int32_t *terms2 = nullptr) {
     // (FP32 holds the values of S and the coefficients, which go with 1 / hi)
     if (!(lo > 1e-30) || !(hi >= lo) || !(hi < 1e30) || hi > 30 * lo) return false;
     const double theta = 0.5 * (hi + lo), delta = std::max(0.5 * (hi - lo), 1e-3 * theta), s1 = theta / delta;
     const double rate = s1 - std::sqrt(s1 * s1 - 1.0);
+    auto terms_for = [&](double target) {
+        int n = 2;
+        while (n < MAX_TERMS && 2 * std::pow(rate, n) > target) ++n;
+        return n;
+    };
     const int passes = std::max(1, (int)std::ceil(std::log(inner_tol) / std::log(3e-7)));
     const double target = std::max(0.5 * std::pow(inner_tol, 1.0 / passes), 1e-7);
-    int terms = 2;
-    while (terms < MAX_TERMS && 2 * std::pow(rate, terms) > target) ++terms;
+    int terms = terms_for(target), second = terms;
     if (2 * std::pow(rate, terms) > target || (terms - 1) * (lowp ? 1 : passes) > inner_max) return false;
+    const double rounding = 1.2e-7 * std::sqrt(hi / lo);
+    if (light > 0.0 && passes == 2) {
+        const int first = terms_for(0.25 * light * inner_tol);
+        const double left = 2 * std::pow(rate, first) + rounding;
+        if (left <= light * inner_tol && first - 1 <= inner_max) {
+            terms = first;
+            second = terms_for(inner_tol / left);
+        }
+    }
     en.terms = terms;
+    if (terms2) *terms2 = second;
     en.inv_theta = (float)(1.0 / theta);
     double rho = 1.0 / s1;
-    for (int k = 1; k < terms; ++k) {
+    for (int k = 1; k < std::max(terms, second); ++k) {
         const double next = 1.0 / (2.0 * s1 - rho);
         en.om[k] = (float)(next * rho);
         en.ga[k] = (float)(2.0 * next / delta);
