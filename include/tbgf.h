@@ -139,7 +139,10 @@ int tb_build_csr(const tb_system_spec *spec, uint64_t seed, tb_bsr *H, tb_bsr *S
                  uint64_t *overlap_seed);
 
 /* ---------------------------------------------------------- sparse product */
-#define TB_PREC_FP64 0  /* all vectors and arithmetic in FP64                      */
+#define TB_PREC_FP64 0  /* all vectors and arithmetic in FP64; with S, the FP32 sweeps
+                           inside the inner solve's refinement (see TB_PREC_DF64)
+                           excepted, whose corrections are checked by, and
+                           repeated until, an FP64 residual below inner_tol    */
 #define TB_PREC_MIXED 1 /* FP32 vectors, SpMM and updates with FP32 accumulation;
                            FP64 recurrence scalars, dot products, convergence
                            tests, projected solutions and reductions           */
@@ -154,8 +157,8 @@ int tb_build_csr(const tb_system_spec *spec, uint64_t seed, tb_bsr *H, tb_bsr *S
                            takes from a short Lanczos run, or conjugate
                            gradients where the spectrum is wide or not
                            positive) and each sweep's c is added to y, t -= S c
-                           with a product in the panel's precision (an FP32 one
-                           once every ||t|| is so small, for the spectrum
+                           with a product in the panel's precision (df panels:
+                           an FP32 one once every ||t|| is so small, for the spectrum
                            of S, that its error stays below inner_tol ||rt|| /
                            20), until ||t|| <=
                            inner_tol ||rt||                                     */

@@ -181,8 +181,8 @@ int run_solver(tb_ctx *ctx, const tb_bsr *H, const tb_bsr *S, const double *z, i
         rc = spectral_bounds(ctx, (const int64_t *)d_srp, (const int32_t *)d_sci, (const double *)d_sval, S->n_brows, b,
                              num_sms(), stream, &lo, &hi);
         if (rc) return rc;
-        const double light = engine_light(lo, hi);
-        engine = chebyshev_terms(lo, hi, inner_tol, inner_max, lowp, en, lowp ? light : 0.0, &en.terms2);
+        const double light = lowp ? engine_light(lo, hi) : 0.0; // FP64: every residual in FP64
+        engine = chebyshev_terms(lo, hi, inner_tol, inner_max, lowp, en, light, &en.terms2);
         en.light = (float)light;
     }
     // slots: the panel width asked for, or 64 (the graph: the next compiled width up to 32, FP32 64); the persistent

@@ -44,3 +44,11 @@ def test_df_passes_in_fp32_only_where_the_spectrum_allows_it():
     r, kappa = _solve(4.0, tb.TB_PREC_DF64)
     assert 9 < kappa < 11                  # 19 between the bounds, which are 5 % of the width outside
     assert r.refinements > 0 and r.light_refinements < 0.1 * r.refinements
+
+
+def test_fp64_passes_are_fp64():
+    """Also where a residual is below the df panels' bound (inner_tol 1e-9: 1.6e-5 after the first sweep)."""
+    r, _ = _solve(1.0, tb.TB_PREC_FP64, inner_tol=1e-9)
+    assert r.refinements > 0 and r.light_refinements == 0
+    r, _ = _solve(1.0, tb.TB_PREC_FP64)
+    assert r.refinements > 0 and r.light_refinements == 0
