@@ -309,7 +309,9 @@ int tb_local_subspaces(const tb_bsr *A, const int64_t *rhs_rows, const int32_t *
  * largest subspace that do not fit a CTA's shared memory, or that leave room for
  * more CTAs when they are elsewhere, are placed in a device workspace of (grid x
  * vectors) instead (read through L2).
- * opts->panel_w is ignored; n_z <= 1024.  Outputs and status as
+ * opts->panel_w is ignored; n_z <= 1024.  Default inner_tol with sweeps (see
+ * TB_PREC_DF64): FP64 max(1e-4 tol, 1e-14), DF64 max(1e-5 tol, 1e-12); with conjugate
+ * gradients max(1e-3 tol, 1e-13; 1e-7 mixed; 1e-12 DF64).  Outputs and status as
  * shifted_cocg_solve.  TB_ERR_SIZE when even the per-shift states and the
  * local block structure do not fit shared memory. */
 int shifted_cocg_solve_local(tb_ctx *ctx, const tb_bsr *H, const tb_bsr *S, const double *z, int32_t n_z,

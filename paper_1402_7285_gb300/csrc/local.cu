@@ -207,15 +207,18 @@ extern "C" int shifted_cocg_solve_local(tb_ctx *ctx, const tb_bsr *H, const tb_b
     LocalArgs2<double> la2;
     std::memset(&la2, 0, sizeof(la2));
     bool sweeps = !mixed;
-    // (the sweeps make the tighter target of the df panel solver cheap here too)
+    // the targets of the sweeps: df as in the panel solver (the sweeps make it cheap).  FP64 a tenth of the conjugate
+    // gradients': those end a small subspace's solve at rounding, far below their target, where the sweeps stop at theirs
+    // (subspaces of 7 atoms, error of G at tol 1e-10: 0.8e-12 with conjugate gradients, 2e-12 with sweeps to 1e-13)
     const double cg_tol = la.inner_tol;
-    if (opts.inner_tol <= 0.0 && lowp && !mixed) la.inner_tol = std::max(1e-5 * opts.tol, 1e-12);
+    if (opts.inner_tol <= 0.0 && !mixed) la.inner_tol = lowp ? std::max(1e-5 * opts.tol, 1e-12) : std::max(1e-4 * opts.tol, 1e-14);
     if (sweeps && has_s) {
         double lo = 1, hi = 0;
         rc = spectral_bounds(ctx, (const int64_t *)d_srp, (const int32_t *)d_sci, (const double *)d_sval, H->n_brows, b,
                              sms, stream, &lo, &hi);
         if (rc) return rc;
-        sweeps = chebyshev_terms(lo, hi, la.inner_tol, la.inner_max, false, la2);
+        sweeps = chebyshev_terms(lo, hi, la.inner_tol, la.inner_max, false, la2) ||
+                 chebyshev_terms(lo, hi, cg_tol, la.inner_max, false, la2); // (as many passes as the target takes)
     }
     if (sweeps) {
         int optin2 = 0;
