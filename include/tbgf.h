@@ -190,7 +190,8 @@ typedef struct {
     int32_t max_iter;    /* outer iterations, default 100000                        */
     int32_t precision;   /* TB_PREC_FP64 (default), TB_PREC_MIXED or TB_PREC_DF64 */
     int32_t panel_w;     /* columns solved together; 0 = 64, or as many as there are
-                            (FP32 panels: the next of 8, 16, 32, 64), autotuned with >= 128
+                            (FP32 panels: the next of 8, 16, 32, 64), or 32 where
+                            the memory does not hold the arrays of more; autotuned with >= 128
                             columns the library times one iteration of its
                             kernels for each width 8..64 and 2 or 3 CTAs per SM
                             and keeps the fastest per column (cached per shape

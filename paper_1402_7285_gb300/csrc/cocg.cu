@@ -225,15 +225,6 @@ int run_solver(tb_ctx *ctx, const tb_bsr *H, const tb_bsr *S, const double *z, i
     const int ncta_fb = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)std::max(1, per_sm - 1) * num_sms(),
                                                                     (H->n_brows + per_cta_f - 1) / per_cta_f));
     const int ncta_max = std::max(std::max(std::max(ncta, ncta_a), ncta_f), engine ? num_sms() * 8 : 0);
-    void *vec_base = nullptr;
-    rc = ws_get(ctx, WS_SOLVE_VEC, vec_bytes * n_vec + (ir ? 3 * vec32_bytes : 0), &vec_base);
-    if (rc == TB_ERR_ALLOC && engine && opts.panel_w == 0 && W > 32) { // half the slots where 64 do not fit
-        tb_solve_opts o = opts;
-        o.panel_w = 32;
-        return run_solver(ctx, H, S, z, n_z, rhs_rows, n_rhs, out_row_ptr, out_rows, &o, G, iters, resid, status,
-                          profile_reps, ms);
-    }
-    if (rc) return rc;
     size_t off = 0;
     auto take = [&](size_t bytes) {
         size_t o = off;
@@ -265,15 +256,23 @@ int run_solver(tb_ctx *ctx, const tb_bsr *H, const tb_bsr *S, const double *z, i
     const size_t o_h32 = lowp ? take(vsz * H->nnzb * bb) : 0;
     const size_t o_s32 = (lowp && has_s) ? take(vsz * S->nnzb * bb) : 0;
     const size_t o_sf32 = ir ? take(sizeof(float) * S->nnzb * bb) : 0; // FP32 S for the sweeps
-    void *small_base = nullptr;
-    rc = ws_get(ctx, WS_SOLVE_SMALL, off, &small_base);
-    if (rc) return rc;
-    char *sb = (char *)small_base;
-    void *proj_base = nullptr;
+    void *vec_base = nullptr, *small_base = nullptr, *proj_base = nullptr;
     const int64_t proj_entries = (int64_t)W * max_col_ent * n_z; // one region of max_col_ent rows per slot
     const bool qmr = opts.solver == TB_SOLVER_QMR;
-    rc = ws_get(ctx, WS_SOLVE_PROJ, sizeof(c64) * (qmr ? 3 : 2) * proj_entries, &proj_base);
+    rc = ws_get(ctx, WS_SOLVE_VEC, vec_bytes * n_vec + (ir ? 3 * vec32_bytes : 0), &vec_base);
+    if (!rc) rc = ws_get(ctx, WS_SOLVE_SMALL, off, &small_base);
+    if (!rc) rc = ws_get(ctx, WS_SOLVE_PROJ, sizeof(c64) * (qmr ? 3 : 2) * proj_entries, &proj_base);
+    if (rc == TB_ERR_ALLOC && engine && opts.panel_w == 0 && W > 32) {
+        // half the slots where 64 do not fit (vectors, or whole solution vectors on the kept rows); what was got
+        // for 64 would be in their way
+        for (int slot : {WS_SOLVE_VEC, WS_SOLVE_SMALL, WS_SOLVE_PROJ}) ws_free(ctx, slot);
+        tb_solve_opts o = opts;
+        o.panel_w = 32;
+        return run_solver(ctx, H, S, z, n_z, rhs_rows, n_rhs, out_row_ptr, out_rows, &o, G, iters, resid, status,
+                          profile_reps, ms);
+    }
     if (rc) return rc;
+    char *sb = (char *)small_base;
 
     TB_CUDA_TRY(ctx, cudaMemsetAsync(sb + o_ctl, 0, sizeof(Ctrl), stream));
     TB_CUDA_TRY(ctx, cudaMemsetAsync(sb + o_stats, 0, sizeof(int64_t) * 4, stream));

@@ -114,6 +114,8 @@ int set_error(tb_ctx *ctx, int code, const char *fmt, ...);
 
 // Device workspace slot `slot` of at least `bytes` (grow-only, owned by ctx).
 int ws_get(tb_ctx *ctx, int slot, size_t bytes, void **out);
+// Gives slot `slot` back.
+void ws_free(tb_ctx *ctx, int slot);
 
 enum WsSlot {
     WS_SPMM_STAGE = 0,  // staging of calls that may return before their work is done (see StageOrder)

@@ -26,13 +26,7 @@ int ws_get(tb_ctx *ctx, int slot, size_t bytes, void **out) {
     }
     bytes = align_up(bytes < 256 ? 256 : bytes, 256);
     if (ctx->ws_size[slot] < bytes) {
-        if (ctx->ws_ptr[slot]) {
-            // earlier work may still read the old buffer
-            cudaDeviceSynchronize();
-            cudaFree(ctx->ws_ptr[slot]);
-            ctx->ws_ptr[slot] = nullptr;
-            ctx->ws_size[slot] = 0;
-        }
+        ws_free(ctx, slot);
         void *p = nullptr;
         cudaError_t e = cudaMalloc(&p, bytes);
         if (e != cudaSuccess) {
@@ -45,6 +39,14 @@ int ws_get(tb_ctx *ctx, int slot, size_t bytes, void **out) {
     }
     *out = ctx->ws_ptr[slot];
     return TB_OK;
+}
+
+void ws_free(tb_ctx *ctx, int slot) {
+    if (slot >= (int)ctx->ws_ptr.size() || !ctx->ws_ptr[slot]) return;
+    cudaDeviceSynchronize(); // earlier work may still read the buffer
+    cudaFree(ctx->ws_ptr[slot]);
+    ctx->ws_ptr[slot] = nullptr;
+    ctx->ws_size[slot] = 0;
 }
 
 static bool capturing(cudaStream_t s) {
