@@ -66,6 +66,10 @@ __device__ __forceinline__ double dot_row(const double *__restrict__ row, const 
     return y;
 }
 
+// Shared memory of the two vectors, or of the sums in their place where those are larger.
+constexpr int EARLY = 5 * (DNT / 32 + 1) + 2 * (DNT / 32); // doubles
+__host__ __device__ constexpr size_t vector_bytes(int64_t maxr) { return 8 * (2 * maxr > EARLY ? 2 * maxr : EARLY); }
+
 template <int B>
 __global__ void __launch_bounds__(DNT) k_desc(const int64_t *__restrict__ h_rp, const int32_t *__restrict__ h_ci,
                                               const double *__restrict__ h_val, const double *__restrict__ s_val,
@@ -73,17 +77,22 @@ __global__ void __launch_bounds__(DNT) k_desc(const int64_t *__restrict__ h_rp, 
                                               const int64_t *__restrict__ sub_ptr,
                                               const int32_t *__restrict__ sub_atoms, int64_t n, int maxa, int dmax,
                                               float *__restrict__ out) {
+    // (no more static shared memory than the kernel ever had, or the largest subspaces would no longer fit: the sums
+    // before the vectors are in use lie in their place)
     extern __shared__ __align__(16) unsigned char smem[];
     const int maxr = maxa * B;
     double *v0 = reinterpret_cast<double *>(smem);
     double *v1 = v0 + maxr;
-    int32_t *atoms = reinterpret_cast<int32_t *>(v1 + maxr);
+    int32_t *atoms = reinterpret_cast<int32_t *>(smem + vector_bytes(maxr));
     int32_t *nbk = atoms + maxa;
     int16_t *nbl = reinterpret_cast<int16_t *>(nbk + maxa * dmax);
     int16_t *cnt = nbl + maxa * dmax;
     int16_t *dist = cnt + maxa;
-    __shared__ double scratch[5][DNT / 32 + 1];
+    typedef double Scratch[DNT / 32 + 1];
+    __shared__ Scratch scratch[2];
     __shared__ int s_shell[6], s_max, s_surf;
+    Scratch *early = reinterpret_cast<Scratch *>(smem);        // [5], then the warps' minima and maxima
+    double *s_mn = reinterpret_cast<double *>(early + 5), *s_mx = s_mn + DNT / 32;
     const int tid = threadIdx.x;
     for (int64_t c = blockIdx.x; c < n; c += gridDim.x) {
         const int64_t a0 = sub_ptr[c];
@@ -165,9 +174,10 @@ __global__ void __launch_bounds__(DNT) k_desc(const int64_t *__restrict__ h_rp, 
             mn = fmin(mn, __shfl_xor_sync(TB_FULL_MASK, mn, o));
             mx = fmax(mx, __shfl_xor_sync(TB_FULL_MASK, mx, o));
         }
-        __shared__ double s_mn[DNT / 32], s_mx[DNT / 32];
         if ((tid & 31) == 0) s_mn[tid >> 5] = mn, s_mx[tid >> 5] = mx;
-        cta_sums(st, scratch);
+        cta_sums(st, early);
+        if (tid == 0)
+            for (int w = 1; w < DNT / 32; ++w) mn = fmin(mn, s_mn[w]), mx = fmax(mx, s_mx[w]);
         const double dmean = st[0] / nrows, dvar = st[1] / nrows - dmean * dmean, hjj = st[2], hrow = st[3], srow = st[4];
         const int dmax_reached = s_max;
         for (int l = tid; l < nat; l += DNT)
@@ -185,8 +195,9 @@ __global__ void __launch_bounds__(DNT) k_desc(const int64_t *__restrict__ h_rp, 
         }
         // --- spectral moments; v_k is zero beyond k hops, so step k takes the rows up to
         // k + 1 hops away and the neighbours up to k (under half of the FP64 products)
-        for (int l = tid; l < nrows; l += DNT) v0[l] = (l == jl) ? 1.0 : 0.0;
         cta_sums(fs, scratch);
+        for (int l = tid; l < nrows; l += DNT) v0[l] = (l == jl) ? 1.0 : 0.0; // (behind the sums in its place)
+        __syncthreads();
         const double fsum = fs[0], fcnt = fs[1];
         double mom[10];
         double *cur = v0, *nxt = v1;
@@ -232,9 +243,8 @@ __global__ void __launch_bounds__(DNT) k_desc(const int64_t *__restrict__ h_rp, 
             o[17] = (float)srow;
             o[18] = (float)dmean;
             o[19] = (float)sqrt(fmax(dvar, 0.0));
-            for (int w = 1; w < DNT / 32; ++w) s_mn[0] = fmin(s_mn[0], s_mn[w]), s_mx[0] = fmax(s_mx[0], s_mx[w]);
-            o[20] = (float)s_mn[0];
-            o[21] = (float)s_mx[0];
+            o[20] = (float)mn;
+            o[21] = (float)mx;
             o[22] = (float)hrow;
             o[23] = (float)(fcnt > 0 ? fsum / fcnt : 0.0);
             o[24] = (float)(nrows / 1000.0);
@@ -299,12 +309,15 @@ extern "C" int tb_descriptors(tb_ctx *ctx, const tb_bsr *H, const tb_bsr *S, con
     if (rc) return rc;
     rc = validate_bsr(ctx, (const int64_t *)drp, (const int32_t *)dci, dval, H->n_brows, H->nnzb, s, "H");
     if (rc) return rc;
-    const size_t sm = (size_t)2 * maxa * b * 8 + (size_t)maxa * 4 + (size_t)maxa * dmax * 6 + (size_t)maxa * 4 + 64;
+    const size_t sm = vector_bytes((int64_t)maxa * b) + (size_t)maxa * 4 + (size_t)maxa * dmax * 6 + (size_t)maxa * 4 + 64;
     int dev = 0, optin = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    TB_CHECK(ctx, sm <= (size_t)optin, TB_ERR_SIZE, "descriptor subspace needs %zu bytes of shared memory", sm);
     const void *fn = b == 1 ? (const void *)k_desc<1> : b == 4 ? (const void *)k_desc<4> : (const void *)k_desc<9>;
+    cudaFuncAttributes at;
+    TB_CUDA_TRY(ctx, cudaFuncGetAttributes(&at, fn));
+    TB_CHECK(ctx, sm + at.sharedSizeBytes <= (size_t)optin, TB_ERR_SIZE, "descriptor subspace needs %zu bytes of shared memory",
+             sm + at.sharedSizeBytes);
     TB_CUDA_TRY(ctx, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     const int grid = (int)std::min<int64_t>(n_rhs, 152 * 4);
 #define TB_DESC_ARGS                                                                                          \
