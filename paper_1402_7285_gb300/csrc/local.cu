@@ -221,8 +221,9 @@ extern "C" int shifted_cocg_solve_local(tb_ctx *ctx, const tb_bsr *H, const tb_b
                  chebyshev_terms(lo, hi, cg_tol, la.inner_max, false, la2); // (as many passes as the target takes)
     }
     if (sweeps) {
-        int optin2 = 0;
+        int optin2 = 0, sm_bytes = 0;
         cudaDeviceGetAttribute(&optin2, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        cudaDeviceGetAttribute(&sm_bytes, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
         LocalLaunch2 L{};
         L.ctx = ctx, L.has_s = has_s, L.sms = sms, L.probe = true;
         if (!(lowp ? launch_local2_df(L, b) : launch_local2_f64(L, b)))
@@ -249,30 +250,40 @@ extern "C" int shifted_cocg_solve_local(tb_ctx *ctx, const tb_bsr *H, const tb_b
         int best = 0;
         for (int mode = 0; mode < 3; ++mode) {
             const size_t sm = fixed + (mode < 2 ? ga : 0) + (mode < 1 ? ow : 0);
-            const int fit = sm > limit ? 0 : (int)std::min<size_t>(1024 / L.threads, (size_t)optin2 / (sm + L.static_bytes + 1024));
+            const int fit = sm > limit ? 0 : (int)std::min<size_t>(1024 / L.threads, (size_t)sm_bytes / (sm + L.static_bytes + 1024)); // (1 KB of the system's)
             if (mode == 2 ? best > 0 : fit <= best) continue;
             best = std::max(fit, 1);
             la2.own_global = mode;
             L.smem = sm;
         }
         if (best == 1 && maxr > 1024) L.threads = 1024;
-        L.grid = (int)std::min<int64_t>(n_rhs, (int64_t)sms * (1024 / L.threads));
-        const size_t o_scr = take(sizeof(c64) * 2 * (size_t)max_kept * n_z * L.grid);
-        const size_t o_gvec = la2.own_global ? take((ow + (la2.own_global == 2 ? ga : 0)) * L.grid) : 0;
-        const size_t o_zc = take(sizeof(c64) * n_z), o_q = take(sizeof(unsigned long long) * 8);
-        const size_t o_h = lowp ? take(sizeof(double) * H->nnzb * bb) : 0;
+        L.grid = (int)std::min<int64_t>(n_rhs, (int64_t)sms * best);
+        const int64_t nv = H->nnzb * bb;
         // FP64 vectors read S's values as the caller has them, in 16-byte loads: from a copy where they do not lie on
         // 16-byte boundaries (H's have to, S's never had to)
         const bool copy_s = !lowp && has_s && ((uintptr_t)d_sval & 15u);
-        const size_t o_s = (lowp && has_s) || copy_s ? take(sizeof(double) * S->nnzb * bb) : 0;
-        const size_t o_sf = has_s ? take(sizeof(float) * S->nnzb * bb) : 0;
+        size_t o_scr, o_gvec, o_zc, o_q, o_h, o_s, o_sf;
         void *wsp = nullptr;
-        rc = ws_get(ctx, WS_SOLVE_SMALL, off, &wsp);
-        if (rc) return rc;
+        for (;;) {
+            off = 0;
+            o_scr = take(sizeof(c64) * 2 * (size_t)max_kept * n_z * L.grid);
+            o_gvec = la2.own_global ? take((ow + (la2.own_global == 2 ? ga : 0)) * L.grid) : 0;
+            o_zc = take(sizeof(c64) * n_z), o_q = take(sizeof(unsigned long long) * 8);
+            o_h = lowp ? take(sizeof(double) * nv) : 0;
+            o_s = (lowp && has_s) || copy_s ? take(sizeof(double) * nv) : 0;
+            o_sf = has_s ? take(sizeof(float) * nv) : 0;
+            rc = ws_get(ctx, WS_SOLVE_SMALL, off, &wsp);
+            // many kept rows and shifts: fewer CTAs where the memory does not hold the solutions of all (k_local has
+            // two to an SM); what is still too much goes to k_local, which needs no FP32 copy of S
+            if (rc != TB_ERR_ALLOC || L.grid <= 2 * sms) break;
+            L.grid = 2 * sms;
+        }
+        if (rc == TB_ERR_ALLOC && has_s) sweeps = false;
+        else if (rc) return rc;
+        if (sweeps) {
         char *ws = (char *)wsp;
         TB_CUDA_TRY(ctx, cudaMemsetAsync(ws + o_q, 0, sizeof(unsigned long long) * 8, stream));
         k_copy_z_local<<<1, 256, 0, stream>>>((const double *)d_z, (c64 *)(ws + o_zc), n_z);
-        const int64_t nv = H->nnzb * bb;
         auto convert = [&](int prec, const void *src, size_t o) {
             if (b == 9 && lowp)
                 convert_values_t(prec, (const double *)src, ws + o, nv, b, stream);
@@ -322,6 +333,7 @@ extern "C" int shifted_cocg_solve_local(tb_ctx *ctx, const tb_bsr *H, const tb_b
         TB_CUDA_TRY(ctx, cudaMemcpyAsync(&fail, la2.fail, sizeof(fail), cudaMemcpyDeviceToHost, stream));
         TB_CUDA_TRY(ctx, cudaStreamSynchronize(stream));
         if (!fail) return finish_call(la.stat);
+        }
     }
 
     la.inner_tol = cg_tol;
