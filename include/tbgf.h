@@ -201,10 +201,16 @@ typedef struct {
                             of the inner solve on S; 0 = max(1e-3 tol, 1e-13) FP64,
                             max(1e-3 tol, 1e-7) mixed, max(1e-5 tol, 1e-12) DF64   */
     int32_t inner_max;   /* S != I: inner iterations per outer iteration (DF64: per
-                            FP32 sweep), 0 = 40                                   */
-    int32_t ctas_per_sm; /* resident CTAs per SM for the panel kernels, 0 = 3;
-                            the FP32 sweep update of the DF64 refinement runs
-                            one fewer (at least 1)                              */
+                            FP32 sweep), 0 = 40.  Chebyshev sweeps take a fixed
+                            number of products for the spectrum of S and
+                            inner_tol: where that is more (FP64 and the local
+                            solver: of all sweeps together) the solve takes
+                            conjugate gradients, which stop there                */
+    int32_t ctas_per_sm; /* resident CTAs per SM for the panel kernels, at most as
+                            many as each is compiled for; 0 = that number (2 or 3)
+                            for the persistent kernel and 3 for the others, of
+                            which the FP32 sweep update of the DF64 refinement
+                            runs one fewer (at least 1)                         */
     void *stream;        /* cudaStream_t to queue work on                         */
     int32_t solver;      /* TB_SOLVER_COCG (default) or TB_SOLVER_QMR                */
     int64_t *stats;      /* optional host array [4]: outer iterations, inner
@@ -242,8 +248,9 @@ void tb_solve_opts_default(tb_solve_opts *opts);
  * iterations run); resid double[n_rhs][n_z] (final recurrence residual
  * ||rt_n|| / |pi^m_n| relative to ||b||); status int32[n_rhs] (TB_COL_*).
  * Method: one seed COCG per column in the S-bilinear form <u,v> = u^T S v
- * (Sec. 3's generalized shifted COCG): p = r + beta p, u = (z_s S - H) p,
- * alpha = r^T S r / p^T u, S r <- S r - alpha u, r = S^-1 (S r) by an inner CG;
+ * (Sec. 3's generalized shifted COCG): p = r + beta p, u = (z_s S - H) p (kept by
+ * u = z_s S r - H r + beta u), alpha = r^T S r / p^T u, S r <- S r - alpha u, r =
+ * S^-1 (S r) by an inner solve (Chebyshev sweeps with refinement, or CG);
  * every shift z_m follows through collinear residuals r_m = r / pi_m, with
  * pi_{n+1} = (1 + alpha_n (z_m - z_s)) pi_n + (alpha_n beta_{n-1} /
  * alpha_{n-1}) (pi_n - pi_{n-1}) and x_m += (alpha_n pi_n / pi_{n+1}) p_m

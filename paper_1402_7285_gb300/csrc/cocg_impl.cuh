@@ -496,13 +496,13 @@ __device__ bool finish_alpha(const Panel<T> &p, int W, const double *red, ColSta
         }
         __syncthreads();
     }
-    // Restart (df panels): a shift's residual is the seed's divided by |pi|, so
-    // a shift much harder than the seed needs the seed residual below what df
-    // carries (about 1e-10).  Once a column's seed residual is below that, its
-    // worst active shift is checked every 512 iterations; if it improved by
-    // less than 1 % the column restarts with that shift as its seed: alpha = 0
-    // this iteration, B / B' reset rt to e_j, C restarts the recurrences;
-    // converged shifts keep their solutions, active ones start from zero.
+    // Restart (df panels): a shift's residual is the seed's divided by |pi|, so a shift
+    // much harder than the seed needs the seed's residual far below the tolerance.  The
+    // column is kept in range there (range_step); should it stagnate all the same, once
+    // the seed residual is below 1e-10 its worst active shift is checked every 512
+    // iterations, and if it improved by less than 1 % the column restarts with that
+    // shift as its seed: alpha = 0 this iteration, B / B' reset rt to e_j, C restarts
+    // the recurrences; converged shifts keep their solutions, active ones start from zero.
     if (p.stall2 > 0.0) {
         const int KM = p.max_col_ent;
         for (int c = threadIdx.x; c < W; c += NT) {

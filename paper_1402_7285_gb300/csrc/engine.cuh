@@ -29,7 +29,8 @@
 // more recurrences), 333, 12 x (87 + 70), 247 + 168 and 74 for rho: 1333 ms a solve of
 // 64 columns at eta 0.5, 685 here.  Small systems are bound by the barriers and their
 // scalar step, 3-8 us a phase: 256 rows x 2 slots FP64 634 -> 120 us an iteration,
-// Anderson 4096 x 32 FP64 81 -> 37.
+// Anderson 4096 x 32 FP64 81 -> 37.  Keeping columns in range (range_step) takes 0.5 us of A
+// and of B there: integer operations on each value of rt and a test per slot.
 // A sweep that does not reduce the residual (bounds that miss part of the spectrum)
 // ends the kernel with fail = 1; the caller then runs the conjugate-gradient path.
 #pragma once
@@ -670,10 +671,8 @@ struct EngineRun {
     }
 
     // ------------------------------------------------------------ refinement pass
-    // mode 0: y = sigma c, t = rt - S y (first pass); 1: y += sigma c, t -= S sigma c;
-    // 2: as 1 with S c and the residual in FP32 (the correction is small, see engine_light).
-    // The pass in FP32 for kernels with the rows of a block in a thread: two slots a
-    // thread halve the loads of S and of the index arrays.
+    // The pass in FP32 (mode 2 of phase_R) for kernels with the rows of a block in a
+    // thread: two slots a thread halve the loads of S and of the index arrays.
     __device__ void phase_R32x2() {
         const Layout g = make_layout(W / 2, 2, units);
         const float *c32 = e.X[e.terms2 & 1];
@@ -717,6 +716,8 @@ struct EngineRun {
         engine_partials<T, 3, 2>(acc, g, p.part, s.sp);
     }
     __device__ __forceinline__ int terms_of(int mode) const { return mode == 0 ? e.terms : e.terms2; }
+    // mode 0: y = sigma c, t = rt - S y (first pass); 1: y += sigma c, t -= S sigma c;
+    // 2: as 1 with S c and the residual in FP32 (the correction is small, see engine_light)
     __device__ void phase_R(int mode) {
         if constexpr (RPT > 1 && HAS_S) {
             if (mode == 2 && W % 2 == 0) return phase_R32x2();
@@ -987,7 +988,11 @@ struct EngineRun {
 };
 
 // CTAs per SM the kernel is compiled for: three when a thread holds the rows of a
-// block (80 registers), two when it holds one row of a system that may be small.
+// block, two when it holds one row of a system that may be small.  At three a thread has
+// 80 registers: k_engine<df, 4, 4, S> spills 1004 bytes of stores and 1116 of loads, <df, 9, 3,
+// S> 928 and 1144 (-Xptxas -v).  The same kernels without S, which have the same A, spill 12 to
+// 32 bytes, so that is R's df product and the FP32 passes.  Two CTAs (128 registers, none
+// spilled) were slower as a whole: A 382 us against 397, X 96 against 82, R in FP32 279 against 227.
 template <int RPT>
 constexpr int engine_ctas() { return RPT > 1 ? 3 : 2; }
 
