@@ -229,7 +229,7 @@ typedef struct {
  *                 sqrt|r_n^T S r_n| / |pi^m_n|, the quasi-norm of the shift's COCG
  *                 residual; equal in exact arithmetic to QMR on the unconjugated
  *                 Lanczos process); a shift stops when its quasi-residual
- *                 tau_n / tau_0 <= tol (resid is that ratio).  No df64 restarts. */
+ *                 tau_n / tau_0 <= tol (resid is that ratio).                     */
 #define TB_SOLVER_COCG 0
 #define TB_SOLVER_QMR 1
 
@@ -263,13 +263,6 @@ void tb_solve_opts_default(tb_solve_opts *opts);
  * power of two, and the pi of its shifts with it, so that a seed that converges
  * long before another shift does not leave the exponents of its vectors; nothing is
  * rounded by that.
- * TB_PREC_DF64 restart: once a column's seed residual ||S r|| is below 1e-10,
- * its worst unconverged shift residual is checked every 512 outer
- * iterations; if it fell by less than 1 % since the previous check, the
- * column restarts with that shift as its new seed: converged shifts keep
- * their results, every unconverged shift starts again from x = 0, and the
- * restart itself takes one outer iteration.  At most two restarts per
- * column; iters counts every iteration run, before and after restarts.
  * Returns TB_OK, or a positive OR of TB_WARN_* when some column did not
  * converge, or a negative error. */
 int shifted_cocg_solve(tb_ctx *ctx, const tb_bsr *H, const tb_bsr *S, const double *z,

@@ -364,8 +364,6 @@ int run_solver(tb_ctx *ctx, const tb_bsr *H, const tb_bsr *S, const double *z, i
     p.part = sb + o_part;
     p.ctl = (Ctrl *)(sb + o_ctl);
     p.tol = opts.tol;
-    // df64 restarts (see k_outer); not with gsQMR, whose smoothing runs over one seed's iterates
-    p.stall2 = (opts.precision == TB_PREC_DF64 && !qmr) ? 1e-20 : 0.0;
     p.inner_tol = inner_tol;
     p.refine_max = 8;
     p.sweep_red = 1e-5;

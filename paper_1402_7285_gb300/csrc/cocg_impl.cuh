@@ -29,7 +29,6 @@ __device__ ColState fresh_column(const Panel<T> &p, int64_t col) {
     C.n_active = p.nz;
     C.in_done = 1;
     C.zs = p.zs;
-    C.chk_n = -1;
     if (col < p.n_cols) {
         C.row = p.col_row[col];
         C.dst = col;
@@ -57,8 +56,7 @@ __device__ __forceinline__ ShiftState fresh_shift() {
     return S;
 }
 
-// A restarting column (a stall restart, or a slot that took the next column of
-// the queue) starts its recurrences again with beta = 0: what it keeps by
+// A slot that took the next column of the queue starts its recurrences again with beta = 0: what it keeps by
 // recurrence (u and p; FP32 panels: p and S p) is cleared, so that nothing of the old
 // column (not even an inf or a NaN) survives the multiplication by zero.
 template <typename T>
@@ -333,8 +331,8 @@ __device__ void pair_step_B(const Panel<T> &p) {
 // With many kept rows per column (full-vector shifted solutions) the pair steps
 // only compute the per-pair coefficients; these kernels apply them to every
 // (column, kept row, shift), shifts fastest, so the FP64 complex arrays stream
-// at full width.  A column that restarts in this iteration (a stall restart or a
-// slot that took the next column) is skipped: A has already cleared its arrays.
+// at full width.  A slot that took the next column in this iteration is skipped: A has
+// already cleared its arrays.
 // k_rows_A (after A): p^m_n = r_n / pi_n + beta^m_{n-1} p^m_{n-1}; gsQMR smoothing.
 // Index of work item t: column c, kept row k, shift m (32-bit division when the
 // work fits, the common case).
@@ -393,7 +391,7 @@ __global__ void k_rows_B(Panel<T> p) {
 
 // End of A (last CTA): alpha_n = rho_n / mu_n from red[2 c], red[2 c + 1] = mu_n of
 // slot c, on the column states col (p.col, or the caller's copy); column completion,
-// retire, refill and restart.  Returns (in every thread) whether some slot's column
+// retire and refill.  Returns (in every thread) whether some slot's column
 // finished.
 template <typename T>
 __device__ bool finish_alpha(const Panel<T> &p, int W, const double *red, ColState *col) {
@@ -496,58 +494,12 @@ __device__ bool finish_alpha(const Panel<T> &p, int W, const double *red, ColSta
         }
         __syncthreads();
     }
-    // Restart (df panels): a shift's residual is the seed's divided by |pi|, so a shift
-    // much harder than the seed needs the seed's residual far below the tolerance.  The
-    // column is kept in range there (range_step); should it stagnate all the same, once
-    // the seed residual is below 1e-10 its worst active shift is checked every 512
-    // iterations, and if it improved by less than 1 % the column restarts with that
-    // shift as its seed: alpha = 0 this iteration, B / B' reset rt to e_j, C restarts
-    // the recurrences; converged shifts keep their solutions, active ones start from zero.
-    if (p.stall2 > 0.0) {
-        const int KM = p.max_col_ent;
-        for (int c = threadIdx.x; c < W; c += NT) {
-            ColState &C = col[c];
-            const bool low = below_stall(C.rn2, C.ex, p.stall2);
-            const int done = C.done, restarts = C.restarts, chk = C.chk_n, its = C.iters;
-            if (done || !low || restarts >= 2) continue;
-            if (chk >= 0 && its - chk < 512) continue;
-            double rw = -1.0;
-            int mw = -1;
-            for (int m = 0; m < p.nz; ++m) {
-                const ShiftState &S = p.sh[(int64_t)c * p.nz + m];
-                if (S.active && S.resid > rw) rw = S.resid, mw = m;
-            }
-            if (mw < 0) continue;
-            if (C.chk_n < 0 || rw < 0.99 * C.chk_w) {
-                C.chk_n = C.iters;
-                C.chk_w = rw;
-                continue;
-            }
-            C.zs = p.z[mw];
-            C.restart = 1;
-            C.restarts += 1;
-            C.chk_n = -1;
-            C.alpha = mk(0.0, 0.0);
-            for (int m = 0; m < p.nz; ++m) {
-                ShiftState &S = p.sh[(int64_t)c * p.nz + m];
-                if (!S.active) continue;
-                S.pi = S.pi_prev = S.pi_next = S.ipi = mk(1.0, 0.0);
-                S.resid = 1.0;
-                for (int k = 0; k < C.n_ent; ++k) {
-                    p.xs[((int64_t)c * KM + k) * p.nz + m] = mk(0.0, 0.0);
-                    p.ps[((int64_t)c * KM + k) * p.nz + m] = mk(0.0, 0.0);
-                }
-            }
-        }
-    }
-    // what this iteration's B scales by (a restarting column's rt becomes e_j)
+    // what this iteration's B scales by (a new column's rt becomes e_j)
     for (int c = threadIdx.x; c < W; c += NT) {
         ColState &C = col[c];
         C.step = C.done || C.restart ? 0 : range_step<T>(C.rn2);
-        if (C.restart) C.ex = 0;
         if (C.step) {
             const double f2 = pow2d(2 * C.step);
-            C.ex += C.step;
             C.rn2 *= f2; // of the vectors as B will leave them
             C.rho = f2 * C.rho;
         }
@@ -656,7 +608,7 @@ __device__ void finish_outer(const Panel<T> &p, int W, const double *rho_next, i
             C.rho = rn;
             continue;
         }
-        if (restart) { // first iteration of the new seed follows
+        if (restart) { // first iteration of the new column follows
             C.beta_prev = C.beta_vec = C.boa = mk(0.0, 0.0);
             C.rho = rn;
             C.restart = 0;

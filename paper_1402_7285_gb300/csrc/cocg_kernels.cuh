@@ -43,22 +43,18 @@ struct ColState {
     int64_t ent0;   // first kept-row entry of the column (index into G's rows)
     int32_t n_ent;  // kept rows of the column
     int32_t fresh;  // 1 from the moment a slot takes a new column until its first iteration ends
-    c64 zs;         // this column's seed shift (changes on a restart)
-    double chk_w;   // worst active shift residual at the last stagnation check
-    int32_t chk_n;  // iteration of that check (-1: none yet)
-    int32_t restarts, restart; // restarts so far; 1 while a restart is in flight
+    c64 zs;         // the seed shift
+    int32_t restart; // 1 while the slot starts a new column of the queue
     int32_t s_bad;  // the inner CG met a direction with d^H S d <= 0 (S not positive definite)
     // inner solve by refinement (df panels): the true residual t = rt - S y in df,
     // FP32 CG sweeps on S c = t, y += c after each sweep
     int32_t in_sweep;   // 1 while this column's inner solve is still refining
     int32_t in_conv;    // 1 once ||t|| <= inner_tol ||rt|| (or the refinement cap is reached)
     int32_t in_refines; // refinements made in this outer iteration
-    int32_t ex;         // the stored rt, r, p, u and pi are 2^ex times the column's own
+    int32_t step;       // B(n) multiplies rt_n by 2^step (see range_step)
     double in_t2;       // ||t||^2 of the true residual at the last refinement
     double in_sig;      // scale of the current FP32 sweep: it solves S c' = t / in_sig
-    // range of the stored vectors (see range_step)
     c64 beta_vec;       // beta_{n-1} 2^step of B(n-1): the factor of the stored p and u in A(n)
-    int32_t step, pad_[3]; // B(n) multiplies rt_n by 2^step (33 doublewords: slots lie in different banks)
 };
 
 // A residual norm usable as a scale (1 when it is zero or not finite).
@@ -89,11 +85,6 @@ __device__ __forceinline__ int range_step(double rn2) {
     if (e >= range_low<T>() || e <= -1023) return 0;
     return (1 - e) / 2; // 2^e <= rn2 < 2^(e + 1), |k| <= 511
 }
-// ||rt||^2 of the column itself below the bound of the stall test (0: never)
-__device__ __forceinline__ bool below_stall(double rn2, int ex, double stall2) {
-    return stall2 > 0.0 && (ex ? (ex > 500 || rn2 * pow2d(-2 * ex) < stall2) : rn2 < stall2);
-}
-
 static_assert(sizeof(ColState) / 8 % 2 == 1, "a thread a slot: no bank conflicts");
 
 struct ShiftState {
@@ -193,7 +184,6 @@ struct Panel {
     cudaGraphConditionalHandle h_outer, h_inner;
     double tol;
     double inner_tol;
-    double stall2;    // seed residual^2 below which a stagnating column restarts (0: never)
     int32_t max_iter;
     int32_t inner_max;
     int64_t outer_cap;

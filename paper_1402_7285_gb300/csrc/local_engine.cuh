@@ -16,7 +16,9 @@
 //    load touches 4-7 lines instead of 18) and rows of 4x4 blocks in 16-byte loads.
 // Seeds that converge long before another shift are kept in range (range_step): on the
 // substitution system (median shift between two bands, 130 draws) 64 calls had columns
-// that broke down without it, 35 with the kernel before.
+// that broke down without it, 35 with the kernel before; and the columns need no restart
+// with another seed (C5's shifts, tol 1e-5, 255 columns: 1160 iterations on average, FP64
+// 1157; with the restarts that made up for lost range before, 1565).
 // Measured (df): fcc b = 4 with overlap, 608 columns of up to 225 atoms, 643 -> 192 ms; b =
 // 9, 152 columns of up to 561 atoms, 445 -> 207 ms, bound by the longest column.  What
 // bounds it: the latency of the block values from L2 (long-scoreboard stalls; b = 9 df
@@ -160,7 +162,7 @@ __global__ void __launch_bounds__(1024) k_local2(const __grid_constant__ LocalAr
 
     typedef typename Acc<T>::P PP;
     __shared__ PP wpart[3][32];
-    __shared__ int s_col, s_jloc, s_nkept, s_nact, s_status, s_stop, s_restart, s_again;
+    __shared__ int s_col, s_jloc, s_nkept, s_nact, s_status, s_stop, s_again;
     __shared__ c64 s_alpha, s_boa, s_beta_prev, s_zs; // s_boa: beta_{n-1} / alpha_{n-1}
     __shared__ double s_rn2;
     __shared__ int s_step;
@@ -170,8 +172,7 @@ __global__ void __launch_bounds__(1024) k_local2(const __grid_constant__ LocalAr
     __shared__ float s_ratio;
     // scalars that only thread 0 uses
     c64 rho = mk(1.0, 0.0);
-    double t2 = 1.0, sig = 1.0, chk_w = 0.0;
-    int chk_n = -1, restarts = 0, ex = 0; // ex: the stored vectors are 2^ex times the column's own
+    double t2 = 1.0, sig = 1.0;
 
     c64 *xs = a.scratch + (int64_t)blockIdx.x * 2 * a.max_kept * a.nz;
     c64 *ps = xs + (int64_t)a.max_kept * a.nz;
@@ -254,7 +255,7 @@ __global__ void __launch_bounds__(1024) k_local2(const __grid_constant__ LocalAr
             s_beta_prev = s_boa = mk(0.0, 0.0);
             s_be = mk<T>(0, 0);
             s_rn2 = 1.0;
-            s_step = ex = 0;
+            s_step = 0;
             t2 = sig = 1.0;
             s_sig = (T)1;
             s_inv = 1;
@@ -276,11 +277,7 @@ __global__ void __launch_bounds__(1024) k_local2(const __grid_constant__ LocalAr
             s_stop = (jloc < 0);
             s_zs = a.zs;
             s_zt = cvt<T>(a.zs);
-            restarts = 0;
-            s_restart = 0;
             s_nact = 0;
-            chk_n = -1;
-            chk_w = 0.0;
         }
         __syncthreads();
 
@@ -410,36 +407,9 @@ __global__ void __launch_bounds__(1024) k_local2(const __grid_constant__ LocalAr
                 mu[1].add(pv.re * u.im);
                 mu[1].add(pv.im * u.re);
             }
-            // Restart with a new seed (df): a shift's residual is the seed's divided by
-            // |pi|, so a shift much harder than the seed needs the seed residual far below
-            // the tolerance.  The column is kept in range there (range_step); should it
-            // stagnate all the same, once the residual is below 1e-10, the worst active shift is checked every 256 iterations; if it improved by less than
-            // 10 % the column restarts with that shift as its seed: converged shifts
-            // keep their solutions, active ones start again from zero.
             sums(mu, [&](double *v) {
                 const int nact = s_nact;
                 s_nact = 0;
-                s_restart = 0;
-                if (nact > 0 && below_stall(s_rn2, ex, a.stall2) && restarts < 2 && (chk_n < 0 || n - chk_n >= 256)) {
-                    int mw = -1;
-                    double rw = -1.0;
-                    for (int m = 0; m < a.nz; ++m)
-                        if (shs[m].active && shs[m].resid > rw) rw = shs[m].resid, mw = m;
-                    if (chk_n >= 0 && mw >= 0 && rw > 0.9 * chk_w) {
-                        s_zs = a.z[mw];
-                        s_zt = cvt<T>(a.z[mw]);
-                        s_restart = 1;
-                        restarts += 1;
-                        chk_n = -1;
-                    } else {
-                        chk_n = n;
-                        chk_w = rw;
-                    }
-                }
-                if (s_restart) {
-                    reset_scalars();
-                    return;
-                }
                 const c64 m = mk(v[0], v[1]);
                 if (nact == 0) {
                     s_stop = 1;
@@ -463,22 +433,6 @@ __global__ void __launch_bounds__(1024) k_local2(const __grid_constant__ LocalAr
                     }
                 }
             });
-            if (s_restart) {
-                for (int m = tid; m < a.nz; m += NTH) {
-                    ShiftL &sm = shs[m];
-                    if (!sm.active) continue;
-                    sm.pi = sm.pi_prev = sm.pi_next = mk(1.0, 0.0);
-                    sm.resid = 1.0;
-                    for (int k = 0; k < s_nkept; ++k) {
-                        xs[(int64_t)k * a.nz + m] = mk(0.0, 0.0);
-                        ps[(int64_t)k * a.nz + m] = mk(0.0, 0.0);
-                    }
-                }
-                reset_vectors();
-                __syncthreads();
-                inner_solve(start);
-                continue; // the next iteration tests the restarted shifts again
-            }
             if (s_stop) break;
             // ---- shifted step B on the last warps: pi_{n+1}, alpha^m, x^m += alpha^m p^m
             const c64 al64 = s_alpha;
@@ -509,7 +463,6 @@ __global__ void __launch_bounds__(1024) k_local2(const __grid_constant__ LocalAr
                 rho = rn;
                 const int k = s_step = range_step<T>(s_rn2); // the vectors and the pi: below
                 if (k) {
-                    ex += k;
                     s_rn2 *= pow2d(2 * k);
                     rho = pow2d(2 * k) * rho;
                 }

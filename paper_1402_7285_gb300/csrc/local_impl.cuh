@@ -48,7 +48,6 @@ struct LocalArgs {
     unsigned long long *queue;
     unsigned long long *stat; // [2]: outer, inner iterations
     double tol, inner_tol;
-    double stall2; // restart threshold on ||rt||^2 (see the restart below); 0 = never
     int32_t max_iter, inner_max;
     c64 *G;
     int32_t *iters;
@@ -142,10 +141,8 @@ __global__ void __launch_bounds__(LNT) k_local(LocalArgs<T> a) {
     __shared__ int s_col, s_nat, s_jloc, s_nkept, s_nact;
     __shared__ c64 s_rho, s_alpha, s_alpha_prev, s_beta_prev;
     __shared__ double s_rn2, s_in_rr, s_in_alpha, s_in_beta, s_in_tol2;
-    __shared__ int s_status, s_stop, s_in_stop, s_restarts, s_restart, s_chk_n;
-    __shared__ double s_chk_w;
+    __shared__ int s_status, s_stop, s_in_stop;
     __shared__ int s_step;
-    int ex = 0; // thread 0: the stored vectors are 2^ex times the column's own
     __shared__ c64 s_zs; // this column's seed shift
 
     const int tid = threadIdx.x;
@@ -219,15 +216,10 @@ __global__ void __launch_bounds__(LNT) k_local(LocalArgs<T> a) {
             s_alpha_prev = mk(1.0, 0.0);
             s_beta_prev = mk(0.0, 0.0);
             s_rn2 = 1.0;
-            ex = 0;
             s_status = TB_COL_MAX_ITER;
             s_stop = (jloc < 0);
             if (jloc < 0) s_status = TB_COL_BREAKDOWN;
             s_zs = a.zs;
-            s_restarts = 0;
-            s_restart = 0;
-            s_chk_n = -1;
-            s_chk_w = 0.0;
         }
         __syncthreads();
 
@@ -353,67 +345,6 @@ __global__ void __launch_bounds__(LNT) k_local(LocalArgs<T> a) {
             }
             if (my_act) atomicAdd(&s_nact, my_act);
             __syncthreads();
-            // Restart with a new seed.  Every shift's residual is the seed's
-            // divided by |pi|: a shift much harder than the seed needs the seed
-            // residual far below the tolerance, below what the working
-            // precision carries (df: near 1e-10 relative).  Once the seed
-            // residual is below that level, the worst active shift is checked
-            // every 256 iterations; if it improved by less than 10 % the column
-            // restarts with that shift as its seed: converged shifts keep their
-            // solutions, active ones start again from zero.
-            if (tid == 0) {
-                s_restart = 0;
-                if (s_nact > 0 && !s_stop && below_stall(s_rn2, ex, a.stall2) && s_restarts < 2 &&
-                    (s_chk_n < 0 || n - s_chk_n >= 256)) {
-                    int mw = -1;
-                    double rw = -1.0;
-                    for (int m = 0; m < a.nz; ++m)
-                        if (shs[m].active && shs[m].resid > rw) rw = shs[m].resid, mw = m;
-                    if (s_chk_n >= 0 && mw >= 0 && rw > 0.9 * s_chk_w) {
-                        s_zs = a.z[mw];
-                        s_restart = 1;
-                        s_restarts += 1;
-                        s_chk_n = -1;
-                    } else {
-                        s_chk_n = n;
-                        s_chk_w = rw;
-                    }
-                }
-            }
-            __syncthreads();
-            if (s_restart) {
-                for (int m = tid; m < a.nz; m += LNT) {
-                    ShiftL &sm = shs[m];
-                    if (!sm.active) continue;
-                    sm.pi = sm.pi_prev = sm.pi_next = mk(1.0, 0.0);
-                    sm.resid = 1.0;
-                    for (int k = 0; k < s_nkept; ++k) {
-                        xs[(int64_t)k * a.nz + m] = mk(0.0, 0.0);
-                        ps[(int64_t)k * a.nz + m] = mk(0.0, 0.0);
-                    }
-                }
-                for (int l = tid; l < nrows; l += LNT) {
-                    const cpx<T> e = mk<T>(l == jloc ? (T)1 : (T)0, 0);
-                    RT[l] = e;
-                    P[l] = mk<T>(0, 0);
-                    U[l] = mk<T>(0, 0);
-                    if constexpr (HAS_S) {
-                        R[l] = e;
-                        SP[l] = mk<T>(0, 0);
-                    }
-                }
-                if (tid == 0) {
-                    s_rho = mk(1.0, 0.0);
-                    s_alpha = mk(0.0, 0.0);
-                    s_alpha_prev = mk(1.0, 0.0);
-                    s_beta_prev = mk(0.0, 0.0);
-                    s_rn2 = 1.0;
-                    ex = 0;
-                }
-                __syncthreads();
-                seed_start();
-                continue; // the next iteration tests the restarted shifts again
-            }
             if (tid == 0) {
                 if (s_nact == 0 && !s_stop) {
                     s_stop = 1;
@@ -528,7 +459,6 @@ __global__ void __launch_bounds__(LNT) k_local(LocalArgs<T> a) {
                 s_rn2 = red[2];
                 const int k = s_step = range_step<T>(s_rn2);
                 if (k) {
-                    ex += k;
                     s_rn2 *= pow2d(2 * k);
                     s_rho = pow2d(2 * k) * s_rho;
                 }
