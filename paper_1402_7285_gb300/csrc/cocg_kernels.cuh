@@ -85,6 +85,7 @@ __device__ __forceinline__ int range_step(double rn2) {
     if (e >= range_low<T>() || e <= -1023) return 0;
     return (1 - e) / 2; // 2^e <= rn2 < 2^(e + 1), |k| <= 511
 }
+
 static_assert(sizeof(ColState) / 8 % 2 == 1, "a thread a slot: no bank conflicts");
 
 struct ShiftState {

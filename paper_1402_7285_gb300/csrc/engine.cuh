@@ -989,9 +989,9 @@ struct EngineRun {
 
 // CTAs per SM the kernel is compiled for: three when a thread holds the rows of a
 // block, two when it holds one row of a system that may be small.  At three a thread has
-// 80 registers: k_engine<df, 4, 4, S> spills 1004 bytes of stores and 1116 of loads, <df, 9, 3,
-// S> 928 and 1144 (-Xptxas -v).  The same kernels without S, which have the same A, spill 12 to
-// 32 bytes, so that is R's df product and the FP32 passes.  Two CTAs (128 registers, none
+// 80 registers: k_engine<df, 4, 4, S> spills 1008 bytes of stores and 1152 of loads, <df, 9, 3,
+// S> 928 and 1176 (-Xptxas -v).  The same kernels without S, which have the same A, spill 12 to
+// 20 bytes, so that is R's df product and the FP32 passes.  Two CTAs (128 registers, none
 // spilled) were slower as a whole: A 382 us against 397, X 96 against 82, R in FP32 279 against 227.
 template <int RPT>
 constexpr int engine_ctas() { return RPT > 1 ? 3 : 2; }

@@ -36,10 +36,12 @@ def test_whole_vectors_in_little_memory(prec):
         want = 32 * slot + 32 * H.n_rows * 48 + (128 << 20)
         assert want < 64 * slot
         fill = torch.empty(free - want, dtype=torch.uint8, device=DEV)
-        r = tb.solve(ctx, Hd, None, z, cols, ptr, kept, precision=prec)
-        with pytest.raises(tb.TbError, match="-3"):  # asked for, they are refused
-            tb.solve(ctx, Hd, None, z, cols, ptr, kept, precision=prec, panel_w=64)
-        del fill
-    torch.cuda.empty_cache()
+        try:
+            r = tb.solve(ctx, Hd, None, z, cols, ptr, kept, precision=prec)
+            with pytest.raises(tb.TbError, match="-3"):  # asked for, they are refused
+                tb.solve(ctx, Hd, None, z, cols, ptr, kept, precision=prec, panel_w=64)
+        finally:
+            del fill
+            torch.cuda.empty_cache()
     assert r.rc == 0 and ref.rc == 0
     assert torch.equal(torch.view_as_real(r.G), torch.view_as_real(ref.G))
